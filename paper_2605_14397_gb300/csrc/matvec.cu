@@ -47,6 +47,16 @@ constexpr int VEC_SLACK = 32;        // elements after xc / tb so rounded-up cop
 struct FF {
     float hi, lo;
 };
+// two FF accumulators side by side, for the packed FP32 instructions
+struct FF2 {
+    float2 hi, lo;
+};
+// Right-hand sides of one F64 pass.  A coefficient costs 11 FP32 operations per F64
+// right-hand side, so from four on the pass is bound by the FP32 pipe and streaming the
+// coefficients again for the next four costs less than the registers of a wider pass:
+// six RHS of a 12,892-element fault (615 MB of coefficients) took 2.82 ms in one pass of a
+// 16-wide kernel that spilled, 0.60 ms in passes of four and two.
+constexpr int F64_PASS = 4;
 
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
@@ -56,45 +66,39 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 
 template <int MODE>
 struct AccT;
-// type: accumulator; vec: output vectors (y, partials); zin: the x / t operands as the
-// kernels read them -- in F64 mode each double is stored pre-split into (hi, lo) floats
-// by the gather and the reduction, so the streaming kernels do no FP64 arithmetic
+// type: accumulator; vec: output vectors (y); part: phase-1 partials as they are stored;
+// zin: the x / t operands as the kernels read them -- in F64 mode each double is stored
+// pre-split into (hi, lo) floats by the gather and the reduction, and the partials are the
+// accumulators themselves, so the streaming kernels do no FP64 arithmetic
 template <>
 struct AccT<0> {
     using type = float;
     using vec = float;
+    using part = float;
     using zin = float;
 };
 template <>
 struct AccT<1> {
     using type = FF;
     using vec = double;
+    using part = float2;
     using zin = float2;
 };
 
-// z operand: one float, or the (hi, lo) split of a double
+// z operand of the F32 mode
 struct Z32 {
     float h;
 };
-struct Z64 {
-    float h, l;
-};
 
 __device__ __forceinline__ Z32 make_z(float v) { return Z32{v}; }
-__device__ __forceinline__ Z64 make_z(float2 v) { return Z64{v.x, v.y}; }
 __device__ __forceinline__ float2 split_d(double v) {
     const float h = (float)v;
     return make_float2(h, (float)(v - (double)h));
 }
-template <class Zin>
-__device__ __forceinline__ Zin zin_zero();
-template <>
-__device__ __forceinline__ float zin_zero<float>() { return 0.f; }
-template <>
-__device__ __forceinline__ float2 zin_zero<float2>() { return make_float2(0.f, 0.f); }
 
 __device__ __forceinline__ void acc_zero(float& a) { a = 0.f; }
-__device__ __forceinline__ void acc_zero(FF& a) { a.hi = 0.f; a.lo = 0.f; }
+__device__ __forceinline__ void acc_zero(FF& a) { a.hi = a.lo = 0.f; }
+__device__ __forceinline__ void acc_zero(FF2& a) { a.hi = a.lo = make_float2(0.f, 0.f); }
 
 __device__ __forceinline__ void acc_fma(float& acc, float a, Z32 z) { acc = fmaf(a, z.h, acc); }
 // two FP32 accumulators against one coefficient: one packed FMA (sm_100-class FFMA2,
@@ -115,13 +119,27 @@ __device__ __forceinline__ void acc_fma_rhs(A* acc, float v, const Z* z, int str
         for (int k = 0; k < NR; ++k) acc_fma(acc[k * stride], v, z[k]);
     }
 }
-__device__ __forceinline__ void acc_fma(FF& acc, float a, Z64 z) {
-    const float p = a * z.h;
-    const float pe = fmaf(a, z.h, -p);
+// one step of the compensated dot product: acc += a (zh + zl)
+__device__ __forceinline__ void ff_fma(float& hi, float& lo, float a, float zh, float zl) {
+    const float p = a * zh;
+    const float pe = fmaf(a, zh, -p);
     float s, e;
-    two_sum(acc.hi, p, s, e);
+    two_sum(hi, p, s, e);
+    hi = s;
+    lo += fmaf(a, zl, e + pe);
+}
+// Two such steps with the packed FP32 instructions of sm_100 (every half rounded like the
+// scalar operation), half the instructions to issue.
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ void ff_fma2(FF2& acc, float2 a, float2 zh, float2 zl) {
+    const float2 p = __fmul2_rn(a, zh);
+    const float2 pe = __ffma2_rn(a, zh, neg2(p));
+    const float2 s = __fadd2_rn(acc.hi, p);
+    const float2 bb = sub2(s, acc.hi);
+    const float2 e = __fadd2_rn(sub2(acc.hi, sub2(s, bb)), sub2(p, bb));
     acc.hi = s;
-    acc.lo += e + pe + a * z.l;
+    acc.lo = __fadd2_rn(acc.lo, __ffma2_rn(a, zl, __fadd2_rn(e, pe)));
 }
 
 __device__ __forceinline__ void acc_add(float& a, float b) { a += b; }
@@ -164,6 +182,11 @@ __device__ __forceinline__ int warp_reduce_scatter(Acc (&acc)[NR], int lane) {
 
 __device__ __forceinline__ float acc_value(float a) { return a; }
 __device__ __forceinline__ double acc_value(const FF& a) { return (double)a.hi + (double)a.lo; }
+// a phase-1 partial as the reduction adds it
+__device__ __forceinline__ float part_value(float a) { return a; }
+__device__ __forceinline__ double part_value(float2 a) { return (double)a.x + (double)a.y; }
+template <class Part>
+using PartSum = decltype(part_value(Part()));
 
 // z operands of one column for NR right-hand sides (p: the column's nr interleaved
 // values in shared memory).  With nr == NR (a multiple of 4 for floats, of 2 for
@@ -186,21 +209,21 @@ __device__ __forceinline__ void load_z(Z32 (&z)[NR], const float* p, int nr) {
 #pragma unroll
     for (int k = 0; k < NR; ++k) z[k] = make_z(k < nr ? p[k] : 0.f);
 }
+// the (hi, lo) operands of one column for NR right-hand sides in F64 mode (16-byte aligned
+// for an even NR)
 template <int NR>
-__device__ __forceinline__ void load_z(Z64 (&z)[NR], const float2* p, int nr) {
+__device__ __forceinline__ void load_z(float2 (&z)[NR], const float2* p) {
     if constexpr (NR % 2 == 0) {
-        if (nr == NR) {
 #pragma unroll
-            for (int q = 0; q < NR / 2; ++q) {
-                const float4 f = reinterpret_cast<const float4*>(p)[q];
-                z[2 * q] = Z64{f.x, f.y};
-                z[2 * q + 1] = Z64{f.z, f.w};
-            }
-            return;
+        for (int q = 0; q < NR / 2; ++q) {
+            const float4 f = reinterpret_cast<const float4*>(p)[q];
+            z[2 * q] = make_float2(f.x, f.y);
+            z[2 * q + 1] = make_float2(f.z, f.w);
         }
-    }
+    } else {
 #pragma unroll
-    for (int k = 0; k < NR; ++k) z[k] = make_z(k < nr ? p[k] : make_float2(0.f, 0.f));
+        for (int k = 0; k < NR; ++k) z[k] = p[k];
+    }
 }
 
 __device__ __forceinline__ float coef(const float* p, int i) { return p[i]; }
@@ -294,10 +317,11 @@ __device__ __forceinline__ uint32_t to_zin(float v, uint32_t*) {
 // per block: the n = r nr entries times G = 128 / n interleaved groups of leaf partials,
 // four independent loads in flight per thread, groups combined in a fixed order.  In F64
 // mode the sums are stored as (hi, lo) float pairs, the form phase 2 reads.
-template <class V, class Zt, bool VEC4>
+template <class Part, class Zt, bool VEC4>
 __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ far, const int32_t* __restrict__ poff,
-                                                   const int32_t* __restrict__ uoff, const V* __restrict__ P,
+                                                   const int32_t* __restrict__ uoff, const Part* __restrict__ P,
                                                    Zt* __restrict__ tb, int nrhs, const int* __restrict__ skip) {
+    using V = PartSum<Part>;
     __shared__ V sp[128];
     pdl_wait();
     pdl_trigger();
@@ -354,12 +378,12 @@ __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ f
             V s0 = 0, s1 = 0, s2 = 0, s3 = 0;
             int q = 0;
             for (; q + 3 < F.n_tleaves; q += 4) {
-                s0 += P[at(q) + e];
-                s1 += P[at(q + 1) + e];
-                s2 += P[at(q + 2) + e];
-                s3 += P[at(q + 3) + e];
+                s0 += part_value(P[at(q) + e]);
+                s1 += part_value(P[at(q + 1) + e]);
+                s2 += part_value(P[at(q + 2) + e]);
+                s3 += part_value(P[at(q + 3) + e]);
             }
-            for (; q < F.n_tleaves; ++q) s0 += P[at(q) + e];
+            for (; q < F.n_tleaves; ++q) s0 += part_value(P[at(q) + e]);
             const Zt t = to_zin((s0 + s1) + (s2 + s3), tb);
             for (int c = 0; c < F.n_sleaves; ++c) tb[(int64_t)uoff[F.ubase + c] * nrhs + e] = t;
         }
@@ -371,12 +395,12 @@ __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ f
     if (g < G) {
         int q = g;
         for (; q + 3 * G < F.n_tleaves; q += 4 * G) {
-            s0 += P[at(q) + e];
-            s1 += P[at(q + G) + e];
-            s2 += P[at(q + 2 * G) + e];
-            s3 += P[at(q + 3 * G) + e];
+            s0 += part_value(P[at(q) + e]);
+            s1 += part_value(P[at(q + G) + e]);
+            s2 += part_value(P[at(q + 2 * G) + e]);
+            s3 += part_value(P[at(q + 3 * G) + e]);
         }
-        for (; q < F.n_tleaves; q += G) s0 += P[at(q) + e];
+        for (; q < F.n_tleaves; q += G) s0 += part_value(P[at(q) + e]);
     }
     sp[threadIdx.x] = (s0 + s1) + (s2 + s3);
     __syncthreads();
@@ -405,13 +429,14 @@ __device__ __forceinline__ int tb16_piece_pos(int64_t l, int q) { return q ^ (in
 // the rank entries, one load fetches 32 offset-table entries which shuffles broadcast.
 // Every block sums its partials in a fixed order.
 constexpr int RED_WARP_LEAVES = 32;
-template <class V, class Zt>
+template <class Part, class Zt>
 __global__ void __launch_bounds__(256) k_reduce_mix(const FarDesc* __restrict__ far,
                                                     const int32_t* __restrict__ poff,
                                                     const int32_t* __restrict__ uoff,
                                                     const int32_t* __restrict__ order, int64_t n_big, int64_t n_all,
-                                                    const V* __restrict__ P, Zt* __restrict__ tb,
+                                                    const Part* __restrict__ P, Zt* __restrict__ tb,
                                                     const int* __restrict__ skip) {
+    using V = PartSum<Part>;
     __shared__ V sp[256];
     constexpr int SPO = 2048;
     __shared__ int32_t spo[SPO];
@@ -433,12 +458,12 @@ __global__ void __launch_bounds__(256) k_reduce_mix(const FarDesc* __restrict__ 
         if (g < G) {
             int q = g;
             for (; q + 3 * G < nt; q += 4 * G) {
-                s0 += P[(int64_t)po[q] + e];
-                s1 += P[(int64_t)po[q + G] + e];
-                s2 += P[(int64_t)po[q + 2 * G] + e];
-                s3 += P[(int64_t)po[q + 3 * G] + e];
+                s0 += part_value(P[(int64_t)po[q] + e]);
+                s1 += part_value(P[(int64_t)po[q + G] + e]);
+                s2 += part_value(P[(int64_t)po[q + 2 * G] + e]);
+                s3 += part_value(P[(int64_t)po[q + 3 * G] + e]);
             }
-            for (; q < nt; q += G) s0 += P[(int64_t)po[q] + e];
+            for (; q < nt; q += G) s0 += part_value(P[(int64_t)po[q] + e]);
         }
         sp[threadIdx.x] = (s0 + s1) + (s2 + s3);
         __syncthreads();
@@ -470,15 +495,15 @@ __global__ void __launch_bounds__(256) k_reduce_mix(const FarDesc* __restrict__ 
                 const int32_t o0 = __shfl_sync(0xffffffffu, mine, q), o1 = __shfl_sync(0xffffffffu, mine, q + 1);
                 const int32_t o2 = __shfl_sync(0xffffffffu, mine, q + 2), o3 = __shfl_sync(0xffffffffu, mine, q + 3);
                 if (on) {
-                    s0 += P[(int64_t)o0 + e];
-                    s1 += P[(int64_t)o1 + e];
-                    s2 += P[(int64_t)o2 + e];
-                    s3 += P[(int64_t)o3 + e];
+                    s0 += part_value(P[(int64_t)o0 + e]);
+                    s1 += part_value(P[(int64_t)o1 + e]);
+                    s2 += part_value(P[(int64_t)o2 + e]);
+                    s3 += part_value(P[(int64_t)o3 + e]);
                 }
             }
             for (; q < m; ++q) {
                 const int32_t o0 = __shfl_sync(0xffffffffu, mine, q);
-                if (on) s0 += P[(int64_t)o0 + e];
+                if (on) s0 += part_value(P[(int64_t)o0 + e]);
             }
         }
         if (on) {
@@ -650,6 +675,21 @@ struct ZRange {
     static constexpr int BYTES = ((MAX_CHUNK_COLS * NR + 2 * ALIGN) * (int)sizeof(V) + 127) / 128 * 128;
 };
 
+// Columns (or column groups) are dealt to the warps round robin through the chunks of a
+// CTA: slot g starts chunk i at column (g - rot) mod G, rot the columns dealt so far.  With
+// every chunk dealt from warp 0 the first warps always got the odd columns -- 53 columns
+// over 16 warps is 4 for five of them and 3 for the rest, so a fifth of the issue slots of
+// the compute-bound variants waited (warps run ahead by the depth of the ring, so the
+// chunks need not balance one by one).
+template <int G>
+__device__ __forceinline__ int deal_start(int g, int rot) {
+    return g >= rot ? g - rot : g - rot + G;
+}
+template <int G>
+__device__ __forceinline__ int deal_next(int rot, int n) {
+    return (rot + n) % G;
+}
+
 // ---- producer: one thread streams this CTA's chunks (and their operands) through the ring
 // (WAIT_T: wait for the preceding kernel -- the reduction producing t -- only before the
 // first chunk whose operand is t; near tiles read x, complete before that kernel began)
@@ -722,6 +762,47 @@ __device__ __forceinline__ void init_ring(uint64_t* full, uint64_t* empty, int n
     __syncthreads();
 }
 
+// The F64 mode's columns of phase 2: c0, c0 + step, ... of a chunk against the NA row
+// blocks of 32 rows this warp holds (col0: the warp's first row of column 0).  NA is a
+// template argument so that the row blocks past a short leaf cost nothing (151-row leaves
+// of a 25,700-triangle mesh: 5 blocks instead of 6).  Scalar operations: packing row
+// blocks in pairs needs a register move for most operands, and took 208 us on those
+// triangles (1.12 GB, 166 us at the copy bandwidth) where this loop takes 197 us and the
+// former one, with address arithmetic per column and 192 rows, 225 us.
+template <int NA, int NR, int RPW, class E>
+__device__ __forceinline__ void ff_columns(FF (&t)[NR][RPW], const E* col0, int ld, const float2* zb, int c0,
+                                           int ncols, int step) {
+    const E* col = col0 + (size_t)c0 * ld;
+    const float2* zc = zb + (size_t)c0 * NR;
+    const int cs = step * ld, zs = step * NR;
+#pragma unroll 2
+    for (int c = c0; c < ncols; c += step, col += cs, zc += zs) {
+        float v[NA];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) v[i] = coef(col, 32 * i);
+        float2 z[NR];
+        load_z<NR>(z, zc);
+#pragma unroll
+        for (int k = 0; k < NR; ++k)
+#pragma unroll
+            for (int i = 0; i < NA; ++i) ff_fma(t[k][i].hi, t[k][i].lo, v[i], z[k].x, z[k].y);
+    }
+}
+// the same for a run-time number of row blocks (1 .. 6)
+template <int NR, int RPW, class E>
+__device__ __forceinline__ void ff_columns_n(FF (&t)[NR][RPW], int nact, const E* col0, int ld, const float2* zb,
+                                             int c0, int ncols, int step) {
+    static_assert(RPW == 6, "one variant per row block count");
+    if (nact == 6)
+        ff_columns<6>(t, col0, ld, zb, c0, ncols, step);
+    else if (nact == 5)
+        ff_columns<5>(t, col0, ld, zb, c0, ncols, step);
+    else if (nact >= 3)
+        ff_columns<4>(t, col0, ld, zb, c0, ncols, step);
+    else if (nact >= 1)
+        ff_columns<2>(t, col0, ld, zb, c0, ncols, step);
+}
+
 // ---- phase 2: y = [D | U] z per row leaf
 // RS > 1 splits each column's rows over RS warps (RPL / RS rows per lane each), so that
 // many right-hand sides fit in registers with more warps in flight.
@@ -786,7 +867,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     Acc acc[NR][RPW];
     float dt[TMT][4];  // TC2: this warp's m-tiles of the leaf (tensor-core part)
     const bool tc16 = TC16 && a.nr == 16;
-    int cur = -1;
+    int cur = -1, rot = 0;
     LeafDesc L{};
 
     auto flush = [&]() {
@@ -890,6 +971,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
         const Zin* zb = (const Zin*)stg + (z0 - (z0 & ~(int64_t)(ZR::ALIGN - 1)));
         const unsigned char* buf = stg + ZR::BYTES;
         const int rows = 3 * L.n;
+        const int cg = deal_start<NG>(g, rot);  // this warp's first column on the CUDA cores
         if constexpr (TC16) {
             if (tc16 && ch.kind != 0) {
                 if (w < TC16_MT && 16 * w < rows) {
@@ -980,9 +1062,21 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
         // accumulators are never flushed, so no bound check is needed per coefficient.
         // With several RHS a warp skips its row blocks past the leaf (leaves of fewer than
         // 64 elements), a warp-uniform test; with one RHS the loop stays branch-free.
+        if constexpr (MODE == 1) {
+            const int nact = max(0, min(RPW, (rows - rbase + 31) >> 5));
+            rot = deal_next<NG>(rot, ch.ncols);
+            if (ch.kind == 0)
+                ff_columns_n(acc, nact, (const float*)buf + rbase + lane, ch.ld, zb, cg, ch.ncols, NG);
+            else
+                ff_columns_n(acc, nact, (const C*)buf + rbase + lane, ch.ld, zb, cg, ch.ncols, NG);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty + s);
+            continue;
+        } else {
         const int nact = NR == 1 ? RPW : max(0, min(RPW, (rows - rbase + 31) >> 5));
-        for (int c = g; c < ch.ncols && nact > 0; c += NG) {
-            decltype(make_z(zin_zero<Zin>())) zv[NR];
+        rot = deal_next<NG>(rot, ch.ncols);
+        for (int c = cg; c < ch.ncols && nact > 0; c += NG) {
+            Z32 zv[NR];
             if constexpr (NR == 1)
                 zv[0] = make_z(zb[c]);
             else
@@ -1007,15 +1101,16 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(empty + s);
+        }
     }
     if (cur >= 0) flush();
 }
 
-// ---- phase 1: P = V_t^T xc_t, one partial per V column
-template <int MODE, class C, int NR, int RPL, int NCW, int ST = STAGES>
+// ---- phase 1: P = V_t^T xc_t, one partial per V column (F32 mode)
+template <class C, int NR, int RPL, int NCW, int ST = STAGES>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
-    using Acc = typename AccT<MODE>::type;
-    using Vv = typename AccT<MODE>::vec;
+    using Acc = float;
+    using Vv = float;
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t* full = (uint64_t*)smem;
     uint64_t* empty = full + ST;
@@ -1043,12 +1138,11 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
     }
     pdl_wait();  // x in cluster order comes from the preceding kernel
     Vv* P = (Vv*)a.out;
-    int cur = -1;
+    int cur = -1, rot = 0;
     int rows = 0;
-    using Zin = typename AccT<MODE>::zin;
-    const Zin* xs = (const Zin*)a.xc;
+    const float* xs = (const float*)a.xc;
     constexpr bool PAIR = std::is_same<C, uint16_t>::value && NR == 1 && RPL == 6;
-    decltype(make_z(zin_zero<Zin>())) xr[NR][RPL];
+    Z32 xr[NR][RPL];
     Chunk nxt = c0 < c1 ? a.chunks[c0] : Chunk{};
     for (int i = c0; i < c1; ++i) {
         const Chunk ch = nxt;
@@ -1065,25 +1159,26 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
                 const int r = PAIR ? 2 * lane + 64 * (ii >> 1) + (ii & 1) : lane + 32 * ii;
 #pragma unroll
                 for (int k = 0; k < NR; ++k)
-                    xr[k][ii] = make_z((r < rows && k < a.nr) ? xs[(3 * (int64_t)L.begin + r) * a.nr + k]
-                                                              : zin_zero<Zin>());
+                    xr[k][ii] = make_z((r < rows && k < a.nr) ? xs[(3 * (int64_t)L.begin + r) * a.nr + k] : 0.f);
             }
         }
         mbar_wait(full + s, (uint32_t)(q / ST) & 1u, a.err, 1, a.wait_ns);
         const C* buf = (const C*)(stage + (size_t)s * STAGE_BYTES);
         if constexpr (NR == 1) {
-            // Four columns (w, w + NCW, w + 2 NCW, w + 3 NCW) per pass: their four warp sums
-            // share one reduce-scatter (6 shuffles instead of 20) and the loads of four
-            // columns are in flight together.
+            // Four neighbouring columns per pass: their four warp sums share one
+            // reduce-scatter (6 shuffles instead of 20) and the loads of four columns are in
+            // flight together.
             // (no per-coefficient bound checks: see the ring zeroing at the kernel start)
             constexpr int CG = 4;
-            for (int c = w; c < ch.ncols; c += CG * NCW) {
+            const int units = (ch.ncols + CG - 1) / CG;
+            for (int u = deal_start<NCW>(w, rot); u < units; u += NCW) {
+                const int c = CG * u;
                 Acc acc[CG];
                 const C* colp[CG];
 #pragma unroll
                 for (int j = 0; j < CG; ++j) {
                     acc_zero(acc[j]);
-                    colp[j] = buf + (size_t)min(c + j * NCW, ch.ncols - 1) * ch.ld;
+                    colp[j] = buf + (size_t)min(c + j, ch.ncols - 1) * ch.ld;
                 }
                 if constexpr (PAIR) {
 #pragma unroll
@@ -1103,14 +1198,17 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
                     }
                 }
                 const int j = warp_reduce_scatter<CG>(acc, lane);
-                const int cj = c + j * NCW;
+                const int cj = c + j;
                 if ((lane & (32 / CG - 1)) == 0 && cj < ch.ncols) P[ch.zoff + cj] = (Vv)acc_value(acc[0]);
             }
+            rot = deal_next<NCW>(rot, units);
             __syncwarp();
             if (lane == 0) mbar_arrive(empty + s);
             continue;
         }
-        for (int c = w; c < ch.ncols; c += NCW) {
+        const int cw = deal_start<NCW>(w, rot);
+        rot = deal_next<NCW>(rot, ch.ncols);
+        for (int c = cw; c < ch.ncols; c += NCW) {
             const C* col = buf + (size_t)c * ch.ld;
             Acc acc[NR];
 #pragma unroll
@@ -1129,6 +1227,131 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
             }
             const int k = warp_reduce_scatter<NR>(acc, lane);
             if ((lane & (32 / NR - 1)) == 0 && k < a.nr) P[(ch.zoff + c) * a.nr + k] = (Vv)acc_value(acc[0]);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty + s);
+    }
+}
+
+// ---- phase 1 in F64 mode (1 to 4 right-hand sides)
+//
+// A warp takes a column at a time, lanes over rows, with four dot products in flight --
+// four columns for one RHS, two for two, one for three or four -- packed in pairs (over
+// the columns for one RHS, over the RHS otherwise) for the packed FP32 instructions; the
+// four sums over the warp share one reduce-scatter.  The leaf's operands stay in registers
+// already split.  Partials are stored as the (hi, lo) accumulators: adding the two in FP64
+// here, with a few lanes active, had kept the FP64 pipe a third busy; the reduction, which
+// waits on memory, does it with full warps.  Rows past a leaf meet x = 0, and NA, the row
+// blocks of 32 the leaf really has, is a template argument of the column loop.
+// Bound by the FP32 pipe and its issue (a packed instruction takes the pipe two cycles, so
+// packing saves issue slots, not pipe time).  One RHS, 25,700 triangles (444 MB of V,
+// 65 us at the copy bandwidth): 116 us with scalar operations over 192 rows, 104 us packed
+// over the leaf's row blocks, 92 us with the columns dealt across chunks (deal_start).
+constexpr int ff_phase1_group(int NR) { return NR == 1 ? 4 : (NR == 2 ? 2 : 1); }  // columns per pass
+template <int NA, int NR, int RPL, class C, class Ld>
+__device__ __forceinline__ void ff_phase1_columns(const float2 (&x)[NR][RPL], const C* buf, int ld, int u0, int ncw,
+                                                  int ncols, int lane, float2* out, Ld load) {
+    constexpr int CG = ff_phase1_group(NR);
+    for (int c = CG * u0; c < ncols; c += CG * ncw) {
+        FF2 acc[2];
+        acc_zero(acc[0]);
+        acc_zero(acc[1]);
+        const C* colp[CG];
+#pragma unroll
+        for (int j = 0; j < CG; ++j) colp[j] = buf + (size_t)min(c + j, ncols - 1) * ld;
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            float v[CG];
+#pragma unroll
+            for (int j = 0; j < CG; ++j) v[j] = load(colp[j], i);
+            if constexpr (NR == 1) {
+                const float2 xh = make_float2(x[0][i].x, x[0][i].x), xl = make_float2(x[0][i].y, x[0][i].y);
+                ff_fma2(acc[0], make_float2(v[0], v[1]), xh, xl);
+                ff_fma2(acc[1], make_float2(v[2], v[3]), xh, xl);
+            } else if constexpr (NR == 2) {
+                const float2 xh = make_float2(x[0][i].x, x[1][i].x), xl = make_float2(x[0][i].y, x[1][i].y);
+                ff_fma2(acc[0], make_float2(v[0], v[0]), xh, xl);
+                ff_fma2(acc[1], make_float2(v[1], v[1]), xh, xl);
+            } else {
+                const float2 vv = make_float2(v[0], v[0]);
+                ff_fma2(acc[0], vv, make_float2(x[0][i].x, x[1][i].x), make_float2(x[0][i].y, x[1][i].y));
+                if constexpr (NR == 4)
+                    ff_fma2(acc[1], vv, make_float2(x[2][i].x, x[3][i].x), make_float2(x[2][i].y, x[3][i].y));
+                else
+                    ff_fma(acc[1].hi.x, acc[1].lo.x, v[0], x[2][i].x, x[2][i].y);
+            }
+        }
+        FF q[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            q[2 * h] = FF{acc[h].hi.x, acc[h].lo.x};
+            q[2 * h + 1] = FF{acc[h].hi.y, acc[h].lo.y};
+        }
+        const int m = warp_reduce_scatter<4>(q, lane);  // value m: column m (one RHS), m / NR (two), RHS m (more)
+        const int cj = c + (NR == 1 ? m : (NR == 2 ? m >> 1 : 0)), k = NR == 1 ? 0 : (NR == 2 ? m & 1 : m);
+        if ((lane & 7) == 0 && cj < ncols && k < NR) out[(int64_t)cj * NR + k] = make_float2(q[0].hi, q[0].lo);
+    }
+}
+
+template <class C, int NR, int RPL, int NCW>
+__global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_f64(StreamArgs a) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t* full = (uint64_t*)smem;
+    uint64_t* empty = full + STAGES;
+    unsigned char* stage = smem + BAR_BYTES;
+    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    {  // finite data behind every unchecked column read, as in k_phase1
+        uint4* z = reinterpret_cast<uint4*>(stage);
+        for (int i = threadIdx.x; i < (STAGES * STAGE_BYTES + P1_TAIL) / 16; i += blockDim.x)
+            z[i] = make_uint4(0u, 0u, 0u, 0u);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the copies write it
+    }
+    init_ring(full, empty, NCW);
+    const int c0 = a.cta_begin[blockIdx.x], c1 = a.cta_begin[blockIdx.x + 1];
+    pdl_trigger();
+    if (w == NCW) {
+        // the V coefficients are constant: the copies start while the gather drains
+        if (lane == 0) produce<C, float2, NR, false>(a, stage, STAGE_BYTES, full, empty, c0, c1);
+        return;
+    }
+    pdl_wait();  // x in cluster order comes from the preceding kernel
+    float2* P = (float2*)a.out;
+    const float2* xs = (const float2*)a.xc;
+    int cur = -1, rows = 0, rot = 0;
+    float2 x[NR][RPL];
+    auto load = [lane](const C* col, int i) { return coef(col, lane + 32 * i); };
+    Chunk nxt = c0 < c1 ? a.chunks[c0] : Chunk{};
+    for (int i = c0; i < c1; ++i) {
+        const Chunk ch = nxt;
+        if (i + 1 < c1) nxt = a.chunks[i + 1];
+        const int q = i - c0, s = q % STAGES;
+        if (ch.leaf != cur) {
+            cur = ch.leaf;
+            const LeafDesc L = a.leaves[cur];
+            rows = 3 * L.n;
+#pragma unroll
+            for (int ii = 0; ii < RPL; ++ii) {
+                const int r = lane + 32 * ii;
+#pragma unroll
+                for (int k = 0; k < NR; ++k)
+                    x[k][ii] = r < rows ? xs[(3 * (int64_t)L.begin + r) * NR + k] : make_float2(0.f, 0.f);
+            }
+        }
+        mbar_wait(full + s, (uint32_t)(q / STAGES) & 1u, a.err, 1, a.wait_ns);
+        const C* buf = (const C*)(stage + (size_t)s * STAGE_BYTES);
+        float2* out = P + ch.zoff * NR;
+        const int u0 = deal_start<NCW>(w, rot);
+        rot = deal_next<NCW>(rot, (ch.ncols + ff_phase1_group(NR) - 1) / ff_phase1_group(NR));
+        if constexpr (RPL == 6) {
+            if (rows <= 128)
+                ff_phase1_columns<4, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, out, load);
+            else if (rows <= 160)
+                ff_phase1_columns<5, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, out, load);
+            else
+                ff_phase1_columns<6, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, out, load);
+        } else {
+            ff_phase1_columns<RPL, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, out, load);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(empty + s);
@@ -1260,7 +1483,6 @@ void timing_accumulate(HMat& H) {
             HM_CUDA(cudaEventElapsedTime(&ms, H.ev[s + i], H.ev[s + i + 1]));
             H.t_acc[i] += ms;
         }
-        ++H.t_count;
     }
     H.ev_used = 0;
 }
@@ -1275,25 +1497,38 @@ void mark(HMat& H, int idx, cudaStream_t st) {
 
 // consumer warps of phase 1 and phase 2, and phase 2's row split, per right-hand-side
 // count: as many warps as the per-thread registers (accumulators and operands) allow
+constexpr int ncw1_for(int NR) { return NR > 4 ? 8 : 16; }
+// F64 mode: six row blocks per warp whatever the leaf size
 template <int MODE>
-constexpr int ncw1_for(int NR) {
-    return NR > 4 ? 8 : 16;
+constexpr int rs_for(int NR, int RPL) {
+    return MODE == 1 ? RPL / 6 : (NR > 4 ? 2 : 1);
 }
-template <int MODE>
-constexpr int ncw2_for(int NR) {
-    return NR > 1 && MODE == 1 ? 8 : 16;
-}
-constexpr int rs_for(int NR) { return NR > 4 ? 2 : 1; }
 
 // ST: ring depth; NCW1V / NCW2V: consumer warps of phase 1 / phase 2 (0: the default for
 // the right-hand-side count).  The tile-shape variants the autotuner chooses from use
 // other values for the single-RHS FP32-vector product.
+// With the producer warp, 16 consumer warps put five warps on one quarter of the SM and
+// leave 96 registers a thread; 15 (14 for an even row split) leave 128, which the 48
+// accumulators and split operands of three or four F64 right-hand sides need.
+template <int MODE>
+constexpr int ncw2_for(int NR, int RS) {
+    return MODE == 1 && NR > 2 ? 16 - RS : 16;
+}
+
 template <int MODE, class C, int NR, int RPL, int ST = STAGES, int NCW1V = 0, int NCW2V = 0>
 void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool timed, cudaStream_t st) {
-    constexpr int NCW = NCW1V ? NCW1V : ncw1_for<MODE>(NR), NCW2 = NCW2V ? NCW2V : ncw2_for<MODE>(NR),
-                  RS = rs_for(NR);
+    constexpr int NCW = NCW1V ? NCW1V : (MODE == 1 ? 16 : ncw1_for(NR)), RS = rs_for<MODE>(NR, RPL),
+                  NCW2 = NCW2V ? NCW2V : ncw2_for<MODE>(NR, RS);
+    static_assert(MODE == 0 || (NR <= F64_PASS && ST == STAGES), "F64 passes");
     using Acc = typename AccT<MODE>::type;
     using V = typename AccT<MODE>::vec;
+    using Part = typename AccT<MODE>::part;
+    auto* const phase1 = [] {
+        if constexpr (MODE == 0)
+            return k_phase1<C, NR, RPL, NCW, ST>;
+        else
+            return k_phase1_f64<C, NR, RPL, NCW>;
+    }();
     const size_t smem1 = BAR_BYTES + (size_t)ST * STAGE_BYTES + P1_TAIL;
     // BF16 factors with 16 RHS on leaves of up to 192 rows: phase 1 on tensor cores
     constexpr bool kTensorPhase1 = MODE == 0 && NR == 16 && std::is_same<C, uint16_t>::value && RPL == 6;
@@ -1301,7 +1536,7 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     // packed BF16 (hi, lo) form (phase 1 stays on the CUDA cores: one mma.sync per 16 x 16
     // tile did not keep up with the stream there)
     constexpr bool kTensorPhase2x1 = MODE == 0 && NR == 1 && std::is_same<C, uint16_t>::value && RPL == 6;
-    static_assert(!kTensorPhase2x1 || (NCW2 == 16 && rs_for(NR) == 1),
+    static_assert(!kTensorPhase2x1 || (NCW2 == 16 && RS == 1),
                   "the single-RHS tensor-core phase 2 assumes 16 consumer warps without row split");
     // BF16 factors with 16 RHS: the U slices of phase 2 on tensor cores as well, reading t
     // in the packed BF16 form of k_reduce_pack16_mix
@@ -1314,8 +1549,7 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     int dev = 0;
     HM_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        HM_CUDA(cudaFuncSetAttribute(k_phase1<MODE, C, NR, RPL, NCW, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem1));
+        HM_CUDA(cudaFuncSetAttribute(phase1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
         if constexpr (kTensorPhase1)
             HM_CUDA(cudaFuncSetAttribute(k_phase1_tc<NCW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
         HM_CUDA(cudaFuncSetAttribute(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST>,
@@ -1332,7 +1566,7 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
         if (tc)
             launch_pdl(k_phase1_tc<NCW>, dim3(H.grid), dim3((NCW + 1) * 32), smem1, st, a);
         else
-            launch_pdl(k_phase1<MODE, C, NR, RPL, NCW, ST>, dim3(H.grid), dim3((NCW + 1) * 32), smem1, st, a);
+            launch_pdl(phase1, dim3(H.grid), dim3((NCW + 1) * 32), smem1, st, a);
         HM_LAUNCH_CHECK();
         if (timed) mark(H, 2, st);
         using Zt = typename AccT<MODE>::zin;
@@ -1341,26 +1575,26 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
         // one RHS: big blocks a CTA each, the others a warp each (red_order)
         const unsigned gm = (unsigned)std::max<int64_t>(1, H.n_red_big + (H.n_red - H.n_red_big + 7) / 8);
         if constexpr (kTensorPhase2x1)
-            launch_pdl(k_reduce_mix<V, uint32_t>, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
+            launch_pdl(k_reduce_mix<Part, uint32_t>, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
                        (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const int32_t*)H.red_order.p,
                        H.n_red_big, H.n_red,
-                       (const V*)a.out, (uint32_t*)base.tb, base.skip);
+                       (const Part*)a.out, (uint32_t*)base.tb, base.skip);
         else if (kTensorPhase2x16 && base.nr == 16)
             launch_pdl(k_reduce_pack16_mix, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
                        (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const int32_t*)H.red_order.p,
                        H.n_red_big, H.n_red, (const float*)a.out, (uint16_t*)base.tb, base.skip);
         else if (base.nr == 1)
-            launch_pdl(k_reduce_mix<V, Zt>, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
+            launch_pdl(k_reduce_mix<Part, Zt>, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
                        (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const int32_t*)H.red_order.p,
                        H.n_red_big, H.n_red,
-                       (const V*)a.out, (Zt*)base.tb, base.skip);
+                       (const Part*)a.out, (Zt*)base.tb, base.skip);
         else if (MODE == 0 && (base.nr & 3) == 0)
-            launch_pdl(k_reduce_tb<V, Zt, MODE == 0>, dim3((unsigned)H.n_far), dim3(128), 0, st,
-                       (const FarDesc*)H.far.p, (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const V*)a.out,
+            launch_pdl(k_reduce_tb<Part, Zt, MODE == 0>, dim3((unsigned)H.n_far), dim3(128), 0, st,
+                       (const FarDesc*)H.far.p, (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const Part*)a.out,
                        (Zt*)base.tb, base.nr, base.skip);
         else
-            launch_pdl(k_reduce_tb<V, Zt, false>, dim3((unsigned)H.n_far), dim3(128), 0, st,
-                       (const FarDesc*)H.far.p, (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const V*)a.out,
+            launch_pdl(k_reduce_tb<Part, Zt, false>, dim3((unsigned)H.n_far), dim3(128), 0, st,
+                       (const FarDesc*)H.far.p, (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const Part*)a.out,
                        (Zt*)base.tb, base.nr, base.skip);
         HM_LAUNCH_CHECK();
         if (timed) mark(H, 3, st);
@@ -1406,12 +1640,22 @@ bool launch_shape_variant(HMat& H, const HMat::Plan& PL, const StreamArgs& a, bo
 
 template <int MODE, class C>
 void launch_nr(HMat& H, const HMat::Plan& PL, const StreamArgs& a, int nrhs, bool timed, cudaStream_t st) {
-    if (nrhs == 1)
-        launch_rpl<MODE, C, 1>(H, PL, a, timed, st);
-    else if (nrhs <= 4)
-        launch_rpl<MODE, C, 4>(H, PL, a, timed, st);
-    else
-        launch_rpl<MODE, C, 16>(H, PL, a, timed, st);
+    if constexpr (MODE == 1) {
+        switch (nrhs) {
+            case 1: return launch_rpl<MODE, C, 1>(H, PL, a, timed, st);
+            case 2: return launch_rpl<MODE, C, 2>(H, PL, a, timed, st);
+            case 3: return launch_rpl<MODE, C, 3>(H, PL, a, timed, st);
+            case 4: return launch_rpl<MODE, C, 4>(H, PL, a, timed, st);
+            default: fail(HM_EINVAL, "product: 1 to 4 right-hand sides per F64 pass");
+        }
+    } else {
+        if (nrhs == 1)
+            launch_rpl<MODE, C, 1>(H, PL, a, timed, st);
+        else if (nrhs <= 4)
+            launch_rpl<MODE, C, 4>(H, PL, a, timed, st);
+        else
+            launch_rpl<MODE, C, 16>(H, PL, a, timed, st);
+    }
 }
 
 // phase 1, reduction and phase 2 on cluster-ordered operands (see hmat_impl.h)
@@ -1606,8 +1850,10 @@ void ensure_product_scratch(HMat& H, int nrhs, cudaStream_t st) {
     H.nrhs_cap = cap;
 }
 
+int product_pass(int dtype) { return dtype == HM_F64 ? F64_PASS : 16; }
+
 void product_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, cudaStream_t st, const int* skip) {
-    if (nr < 1 || nr > 16) fail(HM_EINVAL, "product: 1 to 16 right-hand sides per pass");
+    if (nr < 1 || nr > product_pass(dtype)) fail(HM_EINVAL, "product: too many right-hand sides in one pass");
     ensure_product_scratch(H, nr, st);
     run_core(H, xc, yc, nr, dtype, fac, false, st, skip);
 }
@@ -1621,10 +1867,11 @@ void matvec(HMat& H, const void* x, void* y, int nrhs, int dtype, cudaStream_t s
     // FP32 factors when stored, unless the caller asks for a stored precision
     const int fac = factors == HM_BF16 ? 1 : (factors == HM_F32 ? 0 : (has_factors(H, 0) ? 0 : 1));
     if (!has_factors(H, fac)) fail(HM_EINVAL, "matvec: the requested factor precision is not stored");
-    ensure_product_scratch(H, std::min(nrhs, 16), st);
-    // at most 16 right-hand sides per pass of the coefficient streams
-    for (int k0 = 0; k0 < nrhs; k0 += 16) {
-        const int nr = std::min(16, nrhs - k0);
+    const int pass = product_pass(dtype);
+    ensure_product_scratch(H, std::min(nrhs, pass), st);
+    for (int k0 = 0; k0 < nrhs; k0 += pass) {
+        const int nr = std::min(pass, nrhs - k0);
+        if (H.timing && k0 % 16 == 0) ++H.t_count;  // products of up to 16 right-hand sides
         const int64_t tot = H.ndof * nr;
         const unsigned gb = (unsigned)ceil_div(tot, 256);
         mark(H, 0, st);

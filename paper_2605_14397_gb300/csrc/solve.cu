@@ -1266,8 +1266,12 @@ unsigned g1(int64_t n) { return (unsigned)ceil_div(std::max<int64_t>(n, 1), 256)
 void apply_E(HMat& H, SolveWS& W, const double* z64, const float* z32, void* y, int nr, int dtype, int fac,
              cudaStream_t st, const int* skip = nullptr) {
     if (dtype == HM_F64) {
-        k_interleave_split<<<g1(H.ndof * nr), 256, 0, st>>>(z64, (float2*)W.zi.p, H.ndof, nr);
-        product_core(H, W.zi.p, y, nr, HM_F64, fac, st, skip);
+        const int pass = product_pass(HM_F64);
+        for (int k0 = 0; k0 < nr; k0 += pass) {
+            const int nk = std::min(pass, nr - k0);
+            k_interleave_split<<<g1(H.ndof * nk), 256, 0, st>>>(z64 + k0 * H.ndof, (float2*)W.zi.p, H.ndof, nk);
+            product_core(H, W.zi.p, (double*)y + k0 * H.ndof, nk, HM_F64, fac, st, skip);
+        }
     } else {
         product_core(H, z32, y, nr, HM_F32, fac, st, skip);
     }

@@ -1,0 +1,45 @@
+"""FP64-vector products of 1 to 16 right-hand sides: every pass width (1 to 4, and counts cut
+into several passes) on leaves of every row-block count of the kernels (fewer than 64 rows
+to more than 192) and both factor precisions.
+
+Every right-hand side of a product must match its own single-RHS product, which the stored
+operator checks entry by entry elsewhere.  Bar: both are compensated sums whose error is at
+most about (n u)^2 of the row's absolute sum, u = 2^-24, n the terms one accumulator adds
+(at most 948 columns over 14 warps and their partial sums: n < 100): 4e-11; 1e-11 of the
+absolute sums in the 2-norm is asked.
+"""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2605_14397_gb300 import hmat, synth
+
+pytestmark = pytest.mark.gpu
+
+E, NU = 1.0, 0.25
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("leaf", [8, 21, 43, 64, 110])
+def test_f64_passes_match_single_rhs(leaf, storage):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    el = synth.disk_mesh(20)  # 316 elements: leaves of 5 to 79 elements
+    T = hmat.ClusterTree(el, leaf, 1.0)
+    H = hmat.HMatrix(T, el, E, NU, 1e-6, storage)
+    A = np.abs(O.dense_matrix(el, E, NU))
+    X = synth.rhs_normal(3 * el.N, 31 + leaf, 16)
+    x = torch.from_numpy(X).cuda()
+    one = torch.empty_like(x)
+    for k in range(16):
+        xk, yk = x[k].contiguous(), torch.empty(3 * el.N, dtype=torch.float64, device="cuda")
+        H.matvec(xk, yk)
+        one[k] = yk
+    scale = np.linalg.norm(A @ np.abs(X).T, axis=0)
+    for nrhs in (2, 3, 4, 5, 7, 16):
+        y = torch.empty((nrhs, 3 * el.N), dtype=torch.float64, device="cuda")
+        H.matvec(x[:nrhs].contiguous(), y)
+        err = np.linalg.norm((y - one[:nrhs]).cpu().numpy(), axis=1) / scale[:nrhs]
+        assert err.max() <= 1e-11, (nrhs, err)
+    H.check()
