@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "hmat_impl.h"
@@ -205,169 +206,390 @@ __global__ void __launch_bounds__(512) k_bj_build(const LeafDesc* __restrict__ l
 }
 
 // The same inverse for leaves of at most BJR_ROWS rows, with the matrix held in registers:
-// 512 threads, thread (tr, tc) = (t / 32, t % 32) owns rows tr + 16 a (a < AR) and columns
-// tc + 32 b (b < BC), the tile sized by the largest leaf of the launch.  Gauss-Jordan by
-// in-place sweeps with partial pivoting and no row interchanges: step k picks the unused
-// row p_k with the largest |A[i][k]| (ties: the lowest row) and sweeps on (p_k, k) -- the
-// pivot row divided by the pivot, every other row i minus A[i][k] times it, column k
-// replaced by -A[i][k] / pivot and 1 / pivot.  After n sweeps row p_k holds the
+// 16 warps, of which 15 hold the matrix -- lane tc of warp tr owns rows tr + 15 a (a < AR)
+// and columns tc + 32 b (b < BC), the tile sized by the largest leaf of the launch.
+// Gauss-Jordan by in-place sweeps with partial pivoting and no row interchanges: step k
+// picks the unused row p_k with the largest |A[i][k]| (ties: the lowest row) and sweeps on
+// (p_k, k) -- the pivot row divided by the pivot, every other row i minus A[i][k] times it,
+// column k replaced by -A[i][k] / pivot and 1 / pivot.  After n sweeps row p_k holds the
 // coefficients of unknown k against equations p_0 .. p_(n-1), so A^-1[k][m] = W[p_k][q]
 // with p_q = m.
-// A sweep is one uniform rank-1 update A -= c' r'^T, r' the pivot row over the pivot
-// (r'[k] = 1 / pivot), c' column k (c'[p] = -1), followed by two fix-ups: column k minus
-// its old values, and row p set to r'.  Every warp finds the pivot itself (shuffles over
-// the column in shared memory, the taken rows a bit mask per lane), and the column and
-// the scaled pivot row are double-buffered, so a step needs two barriers.
+//
+// The sweeps go in panels of BJR_PB columns.  The last warp sweeps a panel's own columns in
+// its registers and leaves the multipliers c_k[i] (column k as step k found it), the pivots
+// and their rows; the other warps carry the pivot rows of the remaining columns through the
+// panel (a thread per column), bring the next panel's columns up to date for the last warp,
+// and apply the panel's rank-1 updates to their tiles while it sweeps.  Each entry sees the
+// same fused multiply-adds in the same order as with a sweep of the whole matrix per step,
+// so the inverse keeps its bits; that form took two block barriers and a pivot search in
+// every warp for each step's 72 FMAs a thread (395 instructions).  Now a panel takes four
+// barriers and is bound by the last warp's chain of latencies (argmax, division and update,
+// eight times 1,000 cycles), behind which the others' 8 x AR x BC FMAs a thread hide.  512
+// leaves of 187 rows (four waves of CTAs, one an SM: the matrix fills the registers): 1.05 ms
+// a step at a time, 0.60 ms with panels.
 constexpr int BJR_ROWS = 192;
+constexpr int BJR_PB = 8;
+constexpr int BJR_MW = 15;  // warps that hold the matrix
 
-// Steps k = 32 KB .. 32 KB + 31 of the sweep: column k lives in register column KB, a
-// compile-time index, so only lane k % 32 of each warp touches it.  Returns false when the
-// remaining column has no non-zero entry in an unused row (a singular block), with the
-// same decision in every thread.
-template <int AR, int BC, int KB>
-__device__ __forceinline__ bool bjr_steps(float (&A)[AR][BC], unsigned& used, int n, int t, int tr, int tc,
-                                          float (*colk)[16 * AR], float (*rp)[32 * BC], int* pk, int* pinv,
-                                          int* err) {
-    constexpr int M = (16 * AR + 31) / 32;  // row slots per lane in the pivot search
-    for (int kc = 0; kc < 32; ++kc) {
-        const int k = 32 * KB + kc;
-        if (k >= n) return true;
-        const int buf = k & 1;
-        if (tc == kc) {
+template <int AR, int BC>
+struct BjrShared {
+    static constexpr int R = BJR_MW * AR, CB = 32 * BC;  // rows held (>= CB), columns held
+    __align__(16) float c[2][R][BJR_PB + 4];  // multipliers, row by row
+    __align__(16) float r[BJR_PB][CB];    // scaled pivot rows, as their step applies them
+    float fin[BJR_PB][CB];                // pivot rows: before the panel, then after it
+    __align__(16) float w[2][R][BJR_PB + 4];  // a panel's own columns, row by row (rows 48 B apart:
+                                              // eight lanes' 16-byte reads meet 32 banks)
+    __align__(16) float cp[2][BJR_PB][BJR_PB];  // [k][q]: c_k at the pivot row of step q
+    __align__(16) float pinv[2][BJR_PB];
+    int prow[2][BJR_PB], pwarp[2][BJR_PB], pslot[2][BJR_PB];  // pivot rows: their warp, their place in its tile
+    int bad;
+    int pk[BJR_ROWS], kinv[BJR_ROWS];
+};
+
+// f(I) for the run-time index i in [0, N), I a compile-time constant.  The empty asm keeps the
+// branches apart: merged into one access with a computed index they would push the array
+// they index out of the registers.
+template <int I, int N, class F>
+__device__ __forceinline__ void with_index(int i, const F& f) {
+    if constexpr (I < N) {
+        if (i == I) {
+            asm volatile("" ::"n"(I));
+            f(std::integral_constant<int, I>{});
+        } else {
+            with_index<I + 1, N>(i, f);
+        }
+    }
+}
+
+// Sweeps of the pb columns of the panel at column k0 by one warp, lane l rows l + 32 m.
+// free_row[m]: all ones while row l + 32 m is no pivot row yet, else 0.  Returns false when
+// a column has no non-zero entry in a free row (a singular block).  Its length is a chain of
+// latencies (about 1,000 cycles a step): the lanes divide by their own candidates while the
+// warp's maximum is found.  A rolled loop over rows in shared memory: unrolled over registers, the pivot row
+// and the column need branches or selects, and 30 KB of code run once a panel by one warp.
+template <int AR, int BC>
+__device__ __forceinline__ bool bjr_panel(BjrShared<AR, BC>& S, int buf, int k0, int pb, int lane,
+                                          unsigned (&free_row)[BC]) {
+    float(*w)[BJR_PB + 4] = &S.w[buf][0];
+    int my_p = 0;  // lane q: the pivot row of step q and the pivot's reciprocal
+    float my_pinv = 0.f;
+#pragma unroll 1
+    for (int q = 0; q < pb; ++q) {
+        // pivot: the bits of non-negative floats order like the floats; a NaN never wins
+        float c[BC], cand = 1.f;
+        unsigned key[BC], best = 0u, row = 0u;
 #pragma unroll
-            for (int a = 0; a < AR; ++a) colk[buf][tr + 16 * a] = A[a][KB];
+        for (int m = 0; m < BC; ++m) c[m] = w[lane + 32 * m][q];
+#pragma unroll
+        for (int m = 0; m < BC; ++m) {
+            key[m] = __float_as_uint(c[m]) & 0x7fffffffu & free_row[m];
+            best = max(best, key[m]);
+        }
+#pragma unroll
+        for (int m = BC - 1; m >= 0; --m)
+            if (key[m] == best) {
+                row = lane + 32 * m;
+                cand = c[m];
+            }
+        unsigned top = __reduce_max_sync(0xffffffffu, best);
+        float inv = 1.0f / cand;
+        float4 u[BC], v[BC];
+#pragma unroll
+        for (int m = 0; m < BC; ++m) {
+            const float4* o = reinterpret_cast<const float4*>(&w[lane + 32 * m][0]);
+            u[m] = o[0];
+            v[m] = o[1];
+        }
+        if (top > 0x7f800000u) {
+            best = 0u;
+#pragma unroll
+            for (int m = 0; m < BC; ++m) {
+                if (key[m] > 0x7f800000u) key[m] = 0u;
+                best = max(best, key[m]);
+            }
+#pragma unroll
+            for (int m = BC - 1; m >= 0; --m)
+                if (key[m] == best) {
+                    row = lane + 32 * m;
+                    cand = c[m];
+                }
+            inv = 1.0f / cand;
+            top = __reduce_max_sync(0xffffffffu, best);
+        }
+        if (top == 0u) return false;
+        const int p = (int)__reduce_min_sync(0xffffffffu, best == top ? row : 0xffffffffu);  // ties: the lowest row
+        const float pinv = __shfl_sync(0xffffffffu, inv, p & 31);
+        const float4 r0 = *reinterpret_cast<const float4*>(&w[p][0]), r1 = *reinterpret_cast<const float4*>(&w[p][4]);
+        float r[BJR_PB] = {r0.x * pinv, r0.y * pinv, r0.z * pinv, r0.w * pinv,
+                           r1.x * pinv, r1.y * pinv, r1.z * pinv, r1.w * pinv};
+#pragma unroll
+        for (int j = 0; j < BJR_PB; ++j) r[j] = j == q ? pinv : r[j];
+        if (lane == q) {
+            my_p = p;
+            my_pinv = pinv;
+        }
+        __syncwarp();  // every lane has read row p
+#pragma unroll
+        for (int m = 0; m < BC; ++m) {
+            if (lane + 32 * m == p) free_row[m] = 0u;
+            u[m].x = fmaf(-c[m], r[0], u[m].x);
+            u[m].y = fmaf(-c[m], r[1], u[m].y);
+            u[m].z = fmaf(-c[m], r[2], u[m].z);
+            u[m].w = fmaf(-c[m], r[3], u[m].w);
+            v[m].x = fmaf(-c[m], r[4], v[m].x);
+            v[m].y = fmaf(-c[m], r[5], v[m].y);
+            v[m].z = fmaf(-c[m], r[6], v[m].z);
+            v[m].w = fmaf(-c[m], r[7], v[m].w);
+            float4* o = reinterpret_cast<float4*>(&w[lane + 32 * m][0]);
+            o[0] = u[m];
+            o[1] = v[m];
+        }
+        if (lane == (p & 31)) {  // its owner: row p is r
+            float4* o = reinterpret_cast<float4*>(&w[p][0]);
+            o[0] = make_float4(r[0], r[1], r[2], r[3]);
+            o[1] = make_float4(r[4], r[5], r[6], r[7]);
+        }
+#pragma unroll
+        for (int m = 0; m < BC; ++m) {
+            S.c[buf][lane + 32 * m][q] = c[m];
+            // column q: -c / pivot, left by the sweep with c on top
+            if (lane + 32 * m != p) w[lane + 32 * m][q] = fmaf(-c[m], pinv, c[m]) - c[m];
+        }
+        __syncwarp();
+    }
+    if (lane < pb) {
+        S.prow[buf][lane] = my_p;
+        S.pwarp[buf][lane] = my_p % BJR_MW;
+        S.pslot[buf][lane] = my_p / BJR_MW;
+        S.pinv[buf][lane] = my_pinv;
+        S.pk[k0 + lane] = my_p;
+        S.kinv[my_p] = k0 + lane;
+    }
+    __syncwarp();
+    for (int e = lane; e < BJR_PB * pb; e += 32) {
+        const int q = e / BJR_PB, k = e % BJR_PB;
+        if (k < pb) S.cp[buf][k][q] = S.c[buf][S.prow[buf][q]][k];
+    }
+    return true;
+}
+
+// The last warp: sweeps panel after panel, each from the columns the matrix warps leave.
+template <int AR, int BC>
+__device__ __forceinline__ void bjr_panel_warp(BjrShared<AR, BC>& S, int n, int lane) {
+    unsigned free_row[BC];
+#pragma unroll
+    for (int m = 0; m < BC; ++m) free_row[m] = lane + 32 * m < n ? 0xffffffffu : 0u;
+    for (int k0 = 0, P = 0; k0 < n; k0 += BJR_PB, ++P) {
+        if (P > 0) {
+            __syncthreads();
+            __syncthreads();
+        }
+        __syncthreads();  // the panel's columns are in S.w
+        if (!bjr_panel<AR, BC>(S, P & 1, k0, min(BJR_PB, n - k0), lane, free_row) && lane == 0) S.bad = 1;
+        __syncthreads();  // the panel is swept
+        if (S.bad) return;
+    }
+    __syncthreads();
+    __syncthreads();
+}
+
+// The matrix warps (tr < 15): the updates of every panel.  False for a singular block.
+template <int AR, int BC>
+__device__ __forceinline__ bool bjr_matrix_warps(float (&A)[AR][BC], BjrShared<AR, BC>& S, int n, int t, int tr,
+                                                 int tc) {
+    const int jc = tc % BJR_PB;
+    // whether this lane holds one of the columns of the panel at k0
+    auto holds = [&](int k0) { return tc / BJR_PB == (k0 / BJR_PB) % (32 / BJR_PB) && k0 + jc < n; };
+    // the steps whose pivot row this warp holds, as a mask
+    auto held = [&](int buf, int pb) { return __ballot_sync(0xffffffffu, tc < pb && S.pwarp[buf][tc & 7] == tr); };
+    // the pivot rows this warp holds into S.fin or back
+    auto rows = [&](int buf, int pb, auto out) {
+        for (unsigned mine = held(buf, pb); mine; mine &= mine - 1u) {
+            const int q = __ffs(mine) - 1;
+            float* s = &S.fin[q][tc];
+            with_index<0, AR>(S.pslot[buf][q], [&](auto a) {
+#pragma unroll
+                for (int b = 0; b < BC; ++b) {
+                    if constexpr (decltype(out)::value)
+                        s[32 * b] = A[a.value][b];
+                    else
+                        A[a.value][b] = s[32 * b];
+                }
+            });
+        }
+    };
+    if (holds(0)) {
+#pragma unroll
+        for (int a = 0; a < AR; ++a) S.w[0][tr + BJR_MW * a][jc] = A[a][0];
+    }
+    __syncthreads();
+    __syncthreads();  // panel 0 is swept
+    if (S.bad) return false;
+    for (int k0 = 0, P = 0; k0 < n; k0 += BJR_PB, ++P) {
+        const int buf = P & 1, pb = min(BJR_PB, n - k0);
+        rows(buf, pb, std::true_type{});
+        __syncthreads();
+        // the pivot rows through the panel, a thread per column (past the last step: r = 0)
+        if (t < 32 * BC) {
+            float v[BJR_PB];
+#pragma unroll
+            for (int q = 0; q < BJR_PB; ++q) v[q] = S.fin[q][t];
+#pragma unroll
+            for (int k = 0; k < BJR_PB; ++k) {
+                if (k >= pb) break;
+                const float4* cp = reinterpret_cast<const float4*>(&S.cp[buf][k][0]);
+                const float4 u = cp[0], x = cp[1];
+                const float c[BJR_PB] = {u.x, u.y, u.z, u.w, x.x, x.y, x.z, x.w};
+                const float rk = v[k] * S.pinv[buf][k];
+                S.r[k][t] = rk;
+#pragma unroll
+                for (int q = 0; q < BJR_PB; ++q) v[q] = q == k ? rk : fmaf(-c[q], rk, v[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < BJR_PB; ++q) S.fin[q][t] = v[q];
         }
         __syncthreads();
-        float bv = -1.f;
-        int bi = 0x7fffffff;
+        const int k1 = k0 + BJR_PB;
+        if (k1 < n) {  // this panel is full: the next panel's columns through it first
+            float r[BJR_PB];
 #pragma unroll
-        for (int m = 0; m < M; ++m) {
-            const int i = tc + 32 * m;
-            if (i < n && !((used >> m) & 1u)) {
-                const float v = fabsf(colk[buf][i]);
-                if (v > bv) {  // rows ascend within a lane: the lowest row wins ties
-                    bv = v;
-                    bi = i;
+            for (int k = 0; k < BJR_PB; ++k) r[k] = S.r[k][(k1 + jc) % (32 * BC)];
+            if (holds(k1)) {
+                with_index<0, BC>(k1 / 32, [&](auto b) {
+#pragma unroll
+                    for (int a = 0; a < AR; ++a) {
+                        const float4* cp = reinterpret_cast<const float4*>(&S.c[buf][tr + BJR_MW * a][0]);
+                        const float4 u = cp[0], v = cp[1];
+                        float x = A[a][b.value];
+                        x = fmaf(-u.x, r[0], x);
+                        x = fmaf(-u.y, r[1], x);
+                        x = fmaf(-u.z, r[2], x);
+                        x = fmaf(-u.w, r[3], x);
+                        x = fmaf(-v.x, r[4], x);
+                        x = fmaf(-v.y, r[5], x);
+                        x = fmaf(-v.z, r[6], x);
+                        x = fmaf(-v.w, r[7], x);
+                        S.w[buf ^ 1][tr + BJR_MW * a][jc] = x;
+                    }
+                });
+            }
+            __syncwarp();
+            for (unsigned mine = held(buf, BJR_PB); mine; mine &= mine - 1u) {
+                const int q = __ffs(mine) - 1;
+                if (holds(k1)) S.w[buf ^ 1][S.prow[buf][q]][jc] = S.fin[q][k1 + jc];
+            }
+            __syncthreads();  // the last warp may sweep them
+            // the panel's updates, four steps at a time
+#pragma unroll
+            for (int h = 0; h < BJR_PB; h += 4) {
+                float rb[4][BC];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int b = 0; b < BC; ++b) rb[k][b] = S.r[h + k][tc + 32 * b];
+#pragma unroll
+                for (int a = 0; a < AR; ++a) {
+                    const float4 c4 = *reinterpret_cast<const float4*>(&S.c[buf][tr + BJR_MW * a][h]);
+                    const float c[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+#pragma unroll
+                        for (int b = 0; b < BC; ++b) A[a][b] = fmaf(-c[k], rb[k][b], A[a][b]);
+                }
+            }
+        } else {
+            for (int k = 0; k < pb; ++k) {
+                float rb[BC];
+#pragma unroll
+                for (int b = 0; b < BC; ++b) rb[b] = S.r[k][tc + 32 * b];
+#pragma unroll
+                for (int a = 0; a < AR; ++a) {
+                    const float c = S.c[buf][tr + BJR_MW * a][k];
+#pragma unroll
+                    for (int b = 0; b < BC; ++b) A[a][b] = fmaf(-c, rb[b], A[a][b]);
                 }
             }
         }
+        rows(buf, pb, std::false_type{});
+        if (holds(k0)) {
+            with_index<0, BC>(k0 / 32, [&](auto b) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (ov > bv || (ov == bv && oi < bi)) {
-                bv = ov;
-                bi = oi;
-            }
+                for (int a = 0; a < AR; ++a) A[a][b.value] = S.w[buf][tr + BJR_MW * a][jc];
+            });
         }
-        if (!(bv > 0.f)) {  // every warp sees the same column: a uniform exit
-            if (t == 0) atomicOr(err, 1);
-            return false;
-        }
-        const int p = bi, ap = p >> 4;
-        if (tc == (p & 31)) used |= 1u << (p >> 5);
-        if (t == 0) {
-            pk[k] = p;
-            pinv[p] = k;
-        }
-        if (tr == (p & 15)) {  // the warp of the pivot row: r' = row p / pivot, r'[k] = 1 / pivot
-            const float pinvv = 1.0f / colk[buf][p];
-#pragma unroll
-            for (int a = 0; a < AR; ++a)
-                if (a == ap)
-#pragma unroll
-                    for (int b = 0; b < BC; ++b)
-                        rp[buf][tc + 32 * b] = (b == KB && tc == kc) ? pinvv : A[a][b] * pinvv;
-        }
-        __syncthreads();
-        float r[BC];
-#pragma unroll
-        for (int b = 0; b < BC; ++b) r[b] = rp[buf][tc + 32 * b];
-#pragma unroll
-        for (int a = 0; a < AR; ++a) {
-            const int i = tr + 16 * a;
-            const float c = (i == p) ? -1.f : colk[buf][i];
-#pragma unroll
-            for (int b = 0; b < BC; ++b) A[a][b] = fmaf(-c, r[b], A[a][b]);
-        }
-        if (tc == kc) {  // column k: -c[i] / pivot (the sweep left c[i] on top)
-#pragma unroll
-            for (int a = 0; a < AR; ++a) A[a][KB] -= colk[buf][tr + 16 * a];
-        }
-        if (tr == (p & 15)) {  // row p: r'
-#pragma unroll
-            for (int a = 0; a < AR; ++a)
-                if (a == ap)
-#pragma unroll
-                    for (int b = 0; b < BC; ++b) A[a][b] = r[b];
+        if (k1 < n) {
+            __syncthreads();  // the next panel is swept
+            if (S.bad) return false;
         }
     }
     return true;
 }
 
-template <int AR, int BC, int KB>
-struct BjrSweep {
-    static __device__ __forceinline__ bool run(float (&A)[AR][BC], unsigned& used, int n, int t, int tr, int tc,
-                                               float (*colk)[16 * AR], float (*rp)[32 * BC], int* pk, int* pinv,
-                                               int* err) {
-        if (!bjr_steps<AR, BC, KB>(A, used, n, t, tr, tc, colk, rp, pk, pinv, err)) return false;
-        return BjrSweep<AR, BC, KB + 1>::run(A, used, n, t, tr, tc, colk, rp, pk, pinv, err);
-    }
-};
 template <int AR, int BC>
-struct BjrSweep<AR, BC, BC> {
-    static __device__ __forceinline__ bool run(float (&)[AR][BC], unsigned&, int, int, int, int, float (*)[16 * AR],
-                                               float (*)[32 * BC], int*, int*, int*) {
-        return true;
-    }
-};
-
-template <int AR, int BC>
-__global__ void __launch_bounds__(512, 1) k_bj_build_reg(const LeafDesc* __restrict__ leaves,
-                                                         const int64_t* __restrict__ self_off,
-                                                         const float* __restrict__ near, const double* __restrict__ d,
-                                                         const double* __restrict__ blk, float* __restrict__ binv,
-                                                         const int64_t* __restrict__ binv_off, int* __restrict__ err) {
+__global__ void __launch_bounds__(512, 1) k_bj_build_reg(
+    const LeafDesc* __restrict__ leaves, const int64_t* __restrict__ self_off, const float* __restrict__ near,
+    const double* __restrict__ d, const double* __restrict__ blk, float* __restrict__ binv,
+    const int64_t* __restrict__ binv_off, int* __restrict__ err) {
     extern __shared__ float wsm[];  // n x n staging (row-major): the block, then W
-    __shared__ float colk[2][16 * AR], rp[2][32 * BC];
-    __shared__ int pk[BJR_ROWS], pinv[BJR_ROWS];
+    __shared__ BjrShared<AR, BC> S;
+    static_assert(BJR_MW * AR >= 32 * BC && 32 * BC <= BJR_ROWS, "every row and column has an owner");
     const LeafDesc L = leaves[blockIdx.x];
     const int n = 3 * L.n;
     const int t = threadIdx.x, tr = t >> 5, tc = t & 31;
     const float* E = near + self_off[blockIdx.x];
-    // the leaf's block of E - diag(d) - C^ep, read column by column (coalesced)
-    for (int q = t; q < n * n; q += 512) {
-        const int j = q / n, i = q % n;
-        float v = E[(int64_t)j * L.ld + i];
-        if (i == j) v -= (float)d[3 * (int64_t)L.begin + i];
-        if (blk && i / 3 == j / 3) v -= (float)blk[9 * ((int64_t)L.begin + i / 3) + 3 * (i % 3) + j % 3];
-        wsm[i * n + j] = v;
+    if (t == 0) S.bad = 0;
+    // the leaf's block of E - diag(d) - C^ep, read column by column (coalesced, a column's
+    // loads in flight together)
+#pragma unroll 2
+    for (int j = tr; j < n; j += 16) {
+        float v[BC];
+#pragma unroll
+        for (int u = 0; u < BC; ++u) v[u] = tc + 32 * u < n ? E[(int64_t)j * L.ld + tc + 32 * u] : 0.f;
+#pragma unroll
+        for (int u = 0; u < BC; ++u)
+            if (tc + 32 * u < n) wsm[(tc + 32 * u) * n + j] = v[u];
     }
     __syncthreads();
-    float A[AR][BC];
-#pragma unroll
-    for (int a = 0; a < AR; ++a)
-#pragma unroll
-        for (int b = 0; b < BC; ++b) {
-            const int i = tr + 16 * a, j = tc + 32 * b;
-            A[a][b] = (i < n && j < n) ? wsm[i * n + j] : 0.f;
+    if (t < n) wsm[t * n + t] -= (float)d[3 * (int64_t)L.begin + t];
+    if (blk) {  // (the diagonal of blk is zero)
+        __syncthreads();
+        for (int e = t; e < 9 * L.n; e += 512) {
+            const int el = e / 9, i = 3 * el + e % 9 / 3, j = 3 * el + e % 3;
+            wsm[i * n + j] -= (float)blk[9 * (int64_t)L.begin + e];
         }
-    unsigned used = 0;  // bit m: row tc + 32 m is a pivot row already
-    const bool ok = BjrSweep<AR, BC, 0>::run(A, used, n, t, tr, tc, colk, rp, pk, pinv, err);
-    __syncthreads();  // every thread is past its last read of wsm
-    if (!ok) return;
-#pragma unroll
-    for (int a = 0; a < AR; ++a)
-#pragma unroll
-        for (int b = 0; b < BC; ++b) {
-            const int i = tr + 16 * a, j = tc + 32 * b;
-            if (i < n && j < n) wsm[i * n + j] = A[a][b];
-        }
+    }
     __syncthreads();
+    if (tr < BJR_MW) {
+        float A[AR][BC];
+#pragma unroll
+        for (int a = 0; a < AR; ++a)
+#pragma unroll
+            for (int b = 0; b < BC; ++b) {
+                const int i = tr + BJR_MW * a, j = tc + 32 * b;
+                A[a][b] = (i < n && j < n) ? wsm[i * n + j] : 0.f;
+            }
+        // (a row written to the staging below is its owner's: no other warp reads it)
+        if (bjr_matrix_warps<AR, BC>(A, S, n, t, tr, tc)) {
+#pragma unroll
+            for (int a = 0; a < AR; ++a)
+#pragma unroll
+                for (int b = 0; b < BC; ++b) {
+                    const int i = tr + BJR_MW * a, j = tc + 32 * b;
+                    if (i < n && j < n) wsm[i * n + j] = A[a][b];
+                }
+        }
+    } else {
+        bjr_panel_warp<AR, BC>(S, n, tc);
+    }
+    __syncthreads();
+    if (S.bad) {
+        if (t == 0) atomicOr(err, 1);
+        return;
+    }
     float* out = binv + binv_off[blockIdx.x];
-    for (int q = t; q < n * n; q += 512) {
-        const int c = q / n, rr = q % n;
-        out[(int64_t)c * L.ld + rr] = wsm[pk[rr] * n + pinv[c]];
+    for (int c = tr; c < n; c += 16) {
+        const int q = S.kinv[c];
+        for (int rr = tc; rr < n; rr += 32) out[(int64_t)c * L.ld + rr] = wsm[S.pk[rr] * n + q];
     }
 }
 
@@ -1544,19 +1766,19 @@ void bj_build(HMat& H, SolveWS& W, cudaStream_t st) {
     for (const LeafDesc& L : H.h_leaves) max_rows = std::max(max_rows, 3 * L.n);
     if (max_rows <= BJR_ROWS) {
         const size_t smem = sizeof(float) * (size_t)max_rows * max_rows;
-        // the register tile of the largest leaf: 16 AR rows, 32 BC columns
+        // the register tile of the largest leaf: 15 AR rows, 32 BC columns
         if (max_rows <= 32)
-            bj_build_reg_launch<2, 1>(H, W, smem, st);
+            bj_build_reg_launch<3, 1>(H, W, smem, st);
         else if (max_rows <= 64)
-            bj_build_reg_launch<4, 2>(H, W, smem, st);
+            bj_build_reg_launch<5, 2>(H, W, smem, st);
         else if (max_rows <= 96)
-            bj_build_reg_launch<6, 3>(H, W, smem, st);
+            bj_build_reg_launch<7, 3>(H, W, smem, st);
         else if (max_rows <= 128)
-            bj_build_reg_launch<8, 4>(H, W, smem, st);
+            bj_build_reg_launch<9, 4>(H, W, smem, st);
         else if (max_rows <= 160)
-            bj_build_reg_launch<10, 5>(H, W, smem, st);
+            bj_build_reg_launch<11, 5>(H, W, smem, st);
         else
-            bj_build_reg_launch<12, 6>(H, W, smem, st);
+            bj_build_reg_launch<13, 6>(H, W, smem, st);
         HM_LAUNCH_CHECK();
         int e = 0;
         HM_CUDA(cudaMemcpyAsync(&e, W.err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
