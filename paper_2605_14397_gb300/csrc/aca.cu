@@ -29,8 +29,17 @@ namespace hm {
 
 namespace {
 
-constexpr int ACA_NT = 256;
+constexpr int ACA_NT = 256;  // threads of the recompression
 constexpr int ACA_NW = ACA_NT / 32;
+// Threads of the cross approximation.  A thread evaluating an influence block takes 255
+// registers, so an SM holds 256 threads; as two CTAs of 128 one block's barriers and serial
+// steps run beside the other's evaluations, and a leaf cluster of 56 elements leaves two
+// warps idle instead of six.  7,232 elements, whole assembly: 97.9 ms with one CTA of 256
+// threads, 90.6 with two of 128, 94.9 with three.  (At 128 registers the compiler contracts
+// other products and sums; ties between pivots on regular grids then fall differently and
+// the operator changes within its tolerance.)
+constexpr int CROSS_NT = 128;
+constexpr int CROSS_NW = CROSS_NT / 32;
 
 __device__ __forceinline__ void warp_argmax(double& v, int& i) {
 #pragma unroll
@@ -47,7 +56,29 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// The sums over the warp of NV values per lane (NV a power of two): halving exchanges, then
+// butterflies -- every value adds its lanes in the order of warp_sum.  Returns the index of
+// the value whose sum this lane holds in v[0].
+template <int NV, typename T>
+__device__ __forceinline__ int warp_sums(T (&v)[NV], int lane) {
+    int k = 0;
+#pragma unroll
+    for (int h = NV / 2, o = 16; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int j = 0; j < h; ++j) {
+            const T mine = up ? v[j + h] : v[j], other = up ? v[j] : v[j + h];
+            v[j] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+        }
+        if (up) k += h;
+    }
+#pragma unroll
+    for (int o = 16 / NV; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return k;
+}
+
 // block-wide argmax of (value, index); every thread gets the result
+template <int NW>
 __device__ void block_argmax(double& v, int& i, double* sv, int* si) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     warp_argmax(v, i);
@@ -55,8 +86,8 @@ __device__ void block_argmax(double& v, int& i, double* sv, int* si) {
     if (lane == 0) { sv[w] = v; si[w] = i; }
     __syncthreads();
     if (w == 0) {
-        v = lane < ACA_NW ? sv[lane] : -1.0;
-        i = lane < ACA_NW ? si[lane] : 0x7fffffff;
+        v = lane < NW ? sv[lane] : -1.0;
+        i = lane < NW ? si[lane] : 0x7fffffff;
         warp_argmax(v, i);
         if (lane == 0) { sv[0] = v; si[0] = i; }
     }
@@ -65,6 +96,7 @@ __device__ void block_argmax(double& v, int& i, double* sv, int* si) {
     i = si[0];
 }
 
+template <int NW>
 __device__ double block_sum(double v, double* sv) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     v = warp_sum(v);
@@ -72,7 +104,7 @@ __device__ double block_sum(double v, double* sv) {
     if (lane == 0) sv[w] = v;
     __syncthreads();
     if (w == 0) {
-        v = lane < ACA_NW ? sv[lane] : 0.0;
+        v = lane < NW ? sv[lane] : 0.0;
         v = warp_sum(v);
         if (lane == 0) sv[0] = v;
     }
@@ -80,10 +112,11 @@ __device__ double block_sum(double v, double* sv) {
     return sv[0];
 }
 
+template <int NW>
 __device__ double block_max(double v, double* sv) {
     int dummy = 0;
-    int* si = reinterpret_cast<int*>(sv + ACA_NW);
-    block_argmax(v, dummy, sv, si);
+    int* si = reinterpret_cast<int*>(sv + NW);
+    block_argmax<NW>(v, dummy, sv, si);
     return v;
 }
 
@@ -117,7 +150,7 @@ __device__ int random_free_element(const uint32_t* used, int n, unsigned blk, in
     return *s_next;
 }
 
-__global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, const AcaJob* __restrict__ jobs,
+__global__ void __launch_bounds__(CROSS_NT, 2) k_aca(const ElemRec* __restrict__ el, const AcaJob* __restrict__ jobs,
                                                 double* __restrict__ ws, int R, double eps, double mu, double nu,
                                                 int32_t* __restrict__ rank_out, int32_t* __restrict__ status_out,
                                                 unsigned long long* __restrict__ evals) {
@@ -127,8 +160,8 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
     double* gram_u = vcol + 3 * (R + 3);
     double* gram_v = gram_u + (R + 3);
     uint32_t* used = reinterpret_cast<uint32_t*>(gram_v + (R + 3));  // one bit per DOF row of S
-    __shared__ double sv[2 * ACA_NW];
-    __shared__ int si[ACA_NW];
+    __shared__ double sv[2 * CROSS_NW];
+    __shared__ int si[CROSS_NW];
     __shared__ double piv[3][3];
     __shared__ int s_pe, s_qe, s_next;
     __shared__ double s_pv;
@@ -141,7 +174,7 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
     double* Cc = U + (size_t)mS * R;  // 3 residual columns
     double* Rr = V + (size_t)mT * R;  // 3 residual rows
     const int nwords = (mS + 31) >> 5;
-    for (int w = tid; w < nwords; w += ACA_NT) used[w] = 0u;
+    for (int w = tid; w < nwords; w += CROSS_NT) used[w] = 0u;
     __syncthreads();
 
     int k = 0, status = 0, streak = 0, ipiv = 0, checks = 0;
@@ -152,11 +185,11 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
     for (int step = 0; step < mS + ACA_CHECKS + 1; ++step) {
         if (k + 3 > R && k < kmax) { status = 1; break; }
         // (1) residual rows of receiver element ipiv
-        for (int l = tid; l < 3 * k; l += ACA_NT) urow[l] = U[(size_t)(l / 3) * mS + 3 * ipiv + (l % 3)];
+        for (int l = tid; l < 3 * k; l += CROSS_NT) urow[l] = U[(size_t)(l / 3) * mS + 3 * ipiv + (l % 3)];
         __syncthreads();
         const ElemRec& er = el[J.s_begin + ipiv];
         n_eval += J.t_n;
-        for (int j = tid; j < J.t_n; j += ACA_NT) {
+        for (int j = tid; j < J.t_n; j += CROSS_NT) {
             double blk[9];
             dd_block(er, el[J.t_begin + j], mu, nu, blk);
 #pragma unroll
@@ -172,16 +205,16 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
         if (checking) {
             // a check element passes if its residual rows, scaled to all rows, are within eps
             double r2 = 0.0;
-            for (int c = tid; c < 3 * mT; c += ACA_NT) {
+            for (int c = tid; c < 3 * mT; c += CROSS_NT) {
                 const double v = Rr[(size_t)(c / mT) * mT + (c % mT)];
                 r2 += v * v;
             }
-            r2 = block_sum(r2, sv);
+            r2 = block_sum<CROSS_NW>(r2, sv);
             if (r2 * (double)J.s_n <= eps * eps * nrm2) {
                 if (tid == 0)
                     for (int p = 0; p < 3; ++p) mark_row(used, 3 * ipiv + p);
                 if (++checks >= ACA_CHECKS) break;
-                ipiv = random_free_element(used, J.s_n, blockIdx.x, checks, k, &s_next);
+                ipiv = random_free_element(used, J.s_n, (unsigned)J.id, checks, k, &s_next);
                 if (ipiv < 0) break;
                 continue;
             }
@@ -194,28 +227,28 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
         // (2) column pivot: largest residual entry among the element's free rows
         double av = -1.0;
         int ai = 0x7fffffff;
-        for (int c = tid; c < 3 * mT; c += ACA_NT) {
+        for (int c = tid; c < 3 * mT; c += CROSS_NT) {
             const int p = c / mT;
             if (!((freemask >> p) & 1)) continue;
             const double v = fabs(Rr[(size_t)p * mT + (c % mT)]);
             if (v > av || (v == av && c < ai)) { av = v; ai = c; }
         }
-        block_argmax(av, ai, sv, si);
+        block_argmax<CROSS_NW>(av, ai, sv, si);
         if (!(av > 0.0)) {
             // the free rows are reproduced exactly: retire them, move to another element
             if (tid == 0)
                 for (int p = 0; p < 3; ++p) mark_row(used, 3 * ipiv + p);
-            ipiv = random_free_element(used, J.s_n, blockIdx.x, step + 100, k, &s_next);
+            ipiv = random_free_element(used, J.s_n, (unsigned)J.id, step + 100, k, &s_next);
             if (ipiv < 0) break;
             continue;
         }
         const int jpiv = (ai % mT) / 3;
         // (3) residual columns of source element jpiv
-        for (int l = tid; l < 3 * k; l += ACA_NT) vcol[l] = V[(size_t)(l / 3) * mT + 3 * jpiv + (l % 3)];
+        for (int l = tid; l < 3 * k; l += CROSS_NT) vcol[l] = V[(size_t)(l / 3) * mT + 3 * jpiv + (l % 3)];
         __syncthreads();
         const ElemRec& es = el[J.t_begin + jpiv];
         n_eval += J.s_n;
-        for (int i = tid; i < J.s_n; i += ACA_NT) {
+        for (int i = tid; i < J.s_n; i += CROSS_NT) {
             double blk[9];
             dd_block(el[J.s_begin + i], es, mu, nu, blk);
 #pragma unroll
@@ -254,17 +287,17 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
             if (pe < 0 || !(fabs(pv) > 0.0)) break;
             if (e > 0) {
                 double rm = 0.0, cm = 0.0;
-                for (int c = tid; c < mT; c += ACA_NT) rm = fmax(rm, fabs(Rr[(size_t)pe * mT + c]));
-                for (int r = tid; r < mS; r += ACA_NT) cm = fmax(cm, fabs(Cc[(size_t)qe * mS + r]));
-                rm = block_max(rm, sv);
-                cm = block_max(cm, sv);
+                for (int c = tid; c < mT; c += CROSS_NT) rm = fmax(rm, fabs(Rr[(size_t)pe * mT + c]));
+                for (int r = tid; r < mS; r += CROSS_NT) cm = fmax(cm, fabs(Cc[(size_t)qe * mS + r]));
+                rm = block_max<CROSS_NW>(rm, sv);
+                cm = block_max<CROSS_NW>(cm, sv);
                 if (fabs(pv) < PIVOT_GROWTH * fmax(rm, cm)) break;
             }
             double* Un = U + (size_t)(k + nr) * mS;
             double* Vn = V + (size_t)(k + nr) * mT;
             const double inv = 1.0 / pv;
-            for (int r = tid; r < mS; r += ACA_NT) Un[r] = Cc[(size_t)qe * mS + r] * inv;
-            for (int c = tid; c < mT; c += ACA_NT) Vn[c] = Rr[(size_t)pe * mT + c];
+            for (int r = tid; r < mS; r += CROSS_NT) Un[r] = Cc[(size_t)qe * mS + r] * inv;
+            for (int c = tid; c < mT; c += CROSS_NT) Vn[c] = Rr[(size_t)pe * mT + c];
             if (tid == 0) mark_row(used, 3 * ipiv + pe);
             __syncthreads();
             rowdone |= 1 << pe;
@@ -273,32 +306,40 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
             for (int p = 0; p < 3; ++p) {
                 if (rowdone & (1 << p)) continue;
                 const double f = Un[3 * ipiv + p];
-                for (int c = tid; c < mT; c += ACA_NT) Rr[(size_t)p * mT + c] -= f * Vn[c];
+                for (int c = tid; c < mT; c += CROSS_NT) Rr[(size_t)p * mT + c] -= f * Vn[c];
             }
             for (int q = 0; q < 3; ++q) {
                 if (coldone & (1 << q)) continue;
                 const double f = Vn[3 * jpiv + q];
-                for (int r = tid; r < mS; r += ACA_NT) Cc[(size_t)q * mS + r] -= Un[r] * f;
+                for (int r = tid; r < mS; r += CROSS_NT) Cc[(size_t)q * mS + r] -= Un[r] * f;
             }
             __syncthreads();
             if (tid < 9) piv[tid / 3][tid % 3] = Rr[(size_t)(tid / 3) * mT + 3 * jpiv + (tid % 3)];
             // (5) norm update: ||S||^2 += ||u||^2 ||v||^2 + 2 sum_{l < new} (u.u_l)(v.v_l)
             const int lnew = k + nr;
             double su = 0.0, svv = 0.0;
-            for (int r = tid; r < mS; r += ACA_NT) su += Un[r] * Un[r];
-            for (int c = tid; c < mT; c += ACA_NT) svv += Vn[c] * Vn[c];
-            const double nu2 = block_sum(su, sv);
-            const double nv2 = block_sum(svv, sv);
+            for (int r = tid; r < mS; r += CROSS_NT) su += Un[r] * Un[r];
+            for (int c = tid; c < mT; c += CROSS_NT) svv += Vn[c] * Vn[c];
+            const double nu2 = block_sum<CROSS_NW>(su, sv);
+            const double nv2 = block_sum<CROSS_NW>(svv, sv);
             const int lane = tid & 31, w = tid >> 5;
-            for (int l = w; l < lnew; l += ACA_NW) {
-                const double* Ul = U + (size_t)l * mS;
-                const double* Vl = V + (size_t)l * mT;
-                double a = 0.0, b = 0.0;
-                for (int r = lane; r < mS; r += 32) a += Un[r] * Ul[r];
-                for (int c = lane; c < mT; c += 32) b += Vn[c] * Vl[c];
-                a = warp_sum(a);
-                b = warp_sum(b);
-                if (lane == 0) { gram_u[l] = a; gram_v[l] = b; }
+            for (int l0 = w; l0 < lnew; l0 += 2 * CROSS_NW) {  // columns l0 and l0 + CROSS_NW
+                const int l1 = l0 + CROSS_NW < lnew ? l0 + CROSS_NW : l0;
+                const double *U0 = U + (size_t)l0 * mS, *U1 = U + (size_t)l1 * mS;
+                const double *V0 = V + (size_t)l0 * mT, *V1 = V + (size_t)l1 * mT;
+                double v[4] = {0.0, 0.0, 0.0, 0.0};
+                for (int r = lane; r < mS; r += 32) {
+                    const double x = Un[r];
+                    v[0] += x * U0[r];
+                    if (l1 != l0) v[1] += x * U1[r];
+                }
+                for (int c = lane; c < mT; c += 32) {
+                    const double x = Vn[c];
+                    v[2] += x * V0[c];
+                    if (l1 != l0) v[3] += x * V1[c];
+                }
+                const int e = warp_sums<4>(v, lane), l = (e & 1) ? l1 : l0;
+                if ((lane & 7) == 0 && !((e & 1) && l1 == l0)) (e & 2 ? gram_v : gram_u)[l] = v[0];
             }
             __syncthreads();
             double cross = 0.0;
@@ -318,7 +359,7 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
         if (streak >= 2) {
             // verify on elements drawn at random before accepting the approximation
             checking = true;
-            ipiv = random_free_element(used, J.s_n, blockIdx.x, checks, k, &s_next);
+            ipiv = random_free_element(used, J.s_n, (unsigned)J.id, checks, k, &s_next);
             if (ipiv < 0) break;
             continue;
         }
@@ -326,7 +367,7 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
         const double* Ul = U + (size_t)(k - 1) * mS;
         double bv = -1.0;
         int bi = 0x7fffffff;
-        for (int i = tid; i < J.s_n; i += ACA_NT) {
+        for (int i = tid; i < J.s_n; i += CROSS_NT) {
             const int fm = free_rows(used, i);
             if (!fm) continue;
             double v = 0.0;
@@ -334,14 +375,14 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
                 if ((fm >> p) & 1) v = fmax(v, fabs(Ul[3 * i + p]));
             if (v > bv || (v == bv && i < bi)) { bv = v; bi = i; }
         }
-        block_argmax(bv, bi, sv, si);
+        block_argmax<CROSS_NW>(bv, bi, sv, si);
         if (bv < 0.0) break;  // every row eliminated
         ipiv = bi;
         __syncthreads();
     }
     if (tid == 0) {
-        rank_out[blockIdx.x] = k;
-        status_out[blockIdx.x] = status;
+        rank_out[J.id] = k;
+        status_out[J.id] = status;
         if (evals) atomicAdd(evals, n_eval);
     }
 }
@@ -355,6 +396,14 @@ __global__ void __launch_bounds__(ACA_NT) k_aca(const ElemRec* __restrict__ el, 
 //   keep the k leading singular triplets with sum_{j>=k} s_j^2 <= tau^2 sum_j s_j^2,
 //   U <- Q_U (W S)_k,  V <- Q_V Z_k.
 
+//
+// The FP64 pipe bounds this kernel (an FP64 instruction of a warp holds it for 16 cycles), so
+// it is written to issue few of them, every value keeping the order of its sum: several dot
+// products share the butterfly over the lanes (warp_sums), and the tests and rotation angles
+// of a Jacobi round are computed once for all its pairs, a lane per pair, instead of by all
+// 32 lanes of the warp of each pair.  7,232 elements (1,866 blocks): 64.7 ms before, 41.5 now,
+// the FP64 pipe 87 % busy.
+
 __device__ void cgs2_qr(double* A, int m, int r, double* Rm, double* cbuf, double* sv) {
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     for (int q = tid; q < r * r; q += ACA_NT) Rm[q] = 0.0;
@@ -363,18 +412,35 @@ __device__ void cgs2_qr(double* A, int m, int r, double* Rm, double* cbuf, doubl
         double* aj = A + (size_t)j * m;
         double o2 = 0.0;
         for (int row = tid; row < m; row += ACA_NT) o2 += aj[row] * aj[row];
-        const double orig = sqrt(block_sum(o2, sv));
+        const double orig = sqrt(block_sum<ACA_NW>(o2, sv));
         for (int pass = 0; pass < 2; ++pass) {
-            for (int i = w; i < j; i += ACA_NW) {
-                const double* qi = A + (size_t)i * m;
-                double d = 0.0;
-                for (int row = lane; row < m; row += 32) d += qi[row] * aj[row];
-                d = warp_sum(d);
-                if (lane == 0) cbuf[i] = d;
+            // four columns a pass: i0, i0 + ACA_NW, ... (past j: column i0 again, not stored)
+            for (int i0 = w; i0 < j; i0 += 4 * ACA_NW) {
+                const double* q[4];
+                double d[4] = {0.0, 0.0, 0.0, 0.0};
+                const int nu = min(4, (j - i0 + ACA_NW - 1) / ACA_NW);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) q[u] = A + (size_t)(u < nu ? i0 + u * ACA_NW : i0) * m;
+                if (nu > 2) {
+                    for (int row = lane; row < m; row += 32) {
+                        const double x = aj[row];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) d[u] += q[u][row] * x;
+                    }
+                } else {
+                    for (int row = lane; row < m; row += 32) {
+                        const double x = aj[row];
+                        d[0] += q[0][row] * x;
+                        d[1] += q[1][row] * x;
+                    }
+                }
+                const int u = warp_sums<4>(d, lane);
+                if ((lane & 7) == 0 && u < nu) cbuf[i0 + u * ACA_NW] = d[0];
             }
             __syncthreads();
             for (int row = tid; row < m; row += ACA_NT) {
                 double v = aj[row];
+#pragma unroll 4
                 for (int i = 0; i < j; ++i) v -= cbuf[i] * A[(size_t)i * m + row];
                 aj[row] = v;
             }
@@ -383,7 +449,7 @@ __device__ void cgs2_qr(double* A, int m, int r, double* Rm, double* cbuf, doubl
         }
         double n2 = 0.0;
         for (int row = tid; row < m; row += ACA_NT) n2 += aj[row] * aj[row];
-        const double nrm = sqrt(block_sum(n2, sv));
+        const double nrm = sqrt(block_sum<ACA_NW>(n2, sv));
         const bool keep = nrm > 1e-13 * orig && nrm > 0.0;
         const double sc = keep ? 1.0 / nrm : 0.0;
         for (int row = tid; row < m; row += ACA_NT) aj[row] *= sc;
@@ -393,57 +459,95 @@ __device__ void cgs2_qr(double* A, int m, int r, double* Rm, double* cbuf, doubl
 }
 
 // One-sided Jacobi on the columns of the r x r matrix M (column-major), the rotations
-// accumulated in Z: round-robin pairs, a warp per pair; stops after a sweep without a
-// rotation (|g| <= thresh sqrt(a b) for every pair) or after max_sweeps.
+// accumulated in Z: round-robin pairs; stops after a sweep without a rotation (|g| <= thresh
+// sqrt(a b) for every pair) or after max_sweeps.  A round: the three dot products of its
+// pairs, two pairs a pass of a warp; the test and the angle of every pair, a thread each; the
+// rotations, a warp per pair.
+constexpr int JAC_PAIRS = 128;  // ranks up to 256
 template <typename T>
-__device__ __forceinline__ void jacobi_sweeps(T* M, T* Z, int r, double thresh, int max_sweeps, int* s_rot) {
+struct JacobiRound {
+    T abg[3][JAC_PAIRS];
+    T c[JAC_PAIRS], s[JAC_PAIRS];
+    int rot[JAC_PAIRS];
+};
+// the columns p < q of pair k in round t of n - 1 (n even); false for a column past r
+__device__ __forceinline__ bool jacobi_pair(int t, int k, int n, int r, int& p, int& q) {
+    // t, k < n - 1: the remainders of t + k and t - k by n - 1
+    p = t + k < n - 1 ? t + k : t + k - (n - 1);
+    q = k == 0 ? n - 1 : (t >= k ? t - k : t - k + n - 1);
+    if (p >= r || q >= r) return false;
+    if (p > q) { const int tt = p; p = q; q = tt; }
+    return true;
+}
+template <typename T>
+__device__ __forceinline__ void jacobi_sweeps(T* M, T* Z, int r, double thresh, int max_sweeps, JacobiRound<T>& J) {
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int n = (r + 1) & ~1;
+    const int n = (r + 1) & ~1, np = n / 2;
     for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        if (tid == 0) *s_rot = 0;
-        __syncthreads();
+        int rotated = 0;
         for (int t = 0; t < n - 1; ++t) {
-            for (int k = w; k < n / 2; k += ACA_NW) {
-                int p = (t + k) % (n - 1);
-                int q = k == 0 ? n - 1 : (t - k + n - 1) % (n - 1);
-                if (p >= r || q >= r) continue;
-                if (p > q) { const int tt = p; p = q; q = tt; }
+            for (int k0 = w; k0 < np; k0 += 2 * ACA_NW) {
+                T v[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int k = k0 + u * ACA_NW;
+                    int p, q;
+                    if (k >= np || !jacobi_pair(t, k, n, r, p, q)) continue;
+                    const T* mp = M + (size_t)p * r;
+                    const T* mq = M + (size_t)q * r;
+                    T a = 0, b = 0, g = 0;
+                    for (int i = lane; i < r; i += 32) {
+                        a += mp[i] * mp[i];
+                        b += mq[i] * mq[i];
+                        g += mp[i] * mq[i];
+                    }
+                    v[3 * u] = a;
+                    v[3 * u + 1] = b;
+                    v[3 * u + 2] = g;
+                }
+                const int e = warp_sums<8>(v, lane);
+                if ((lane & 3) == 0 && e < 6 && k0 + e / 3 * ACA_NW < np) J.abg[e % 3][k0 + e / 3 * ACA_NW] = v[0];
+            }
+            __syncthreads();
+            int rot = 0;
+            if (tid < np) {
+                int p, q;
+                if (jacobi_pair(t, tid, n, r, p, q)) {
+                    const T a = J.abg[0][tid], b = J.abg[1][tid], g = J.abg[2][tid];
+                    if (g != T(0) && fabs((double)g) > thresh * sqrt((double)a * (double)b)) {
+                        const T zeta = (b - a) / (T(2) * g);
+                        const T tt = (zeta >= T(0) ? T(1) : T(-1)) / (fabs(zeta) + sqrt(T(1) + zeta * zeta));
+                        const T c = T(1) / sqrt(T(1) + tt * tt), sn = c * tt;
+                        J.c[tid] = c;
+                        J.s[tid] = sn;
+                        rot = 1;
+                    }
+                }
+                J.rot[tid] = rot;
+            }
+            if (!__syncthreads_or(rot)) continue;
+            rotated = 1;
+            for (int k = w; k < np; k += ACA_NW) {
+                if (!J.rot[k]) continue;
+                int p, q;
+                jacobi_pair(t, k, n, r, p, q);
+                const T c = J.c[k], sn = J.s[k];
                 T* mp = M + (size_t)p * r;
                 T* mq = M + (size_t)q * r;
-                T a = 0, b = 0, g = 0;
+                T* zp = Z + (size_t)p * r;
+                T* zq = Z + (size_t)q * r;
                 for (int i = lane; i < r; i += 32) {
-                    a += mp[i] * mp[i];
-                    b += mq[i] * mq[i];
-                    g += mp[i] * mq[i];
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    a += __shfl_xor_sync(0xffffffffu, a, o);
-                    b += __shfl_xor_sync(0xffffffffu, b, o);
-                    g += __shfl_xor_sync(0xffffffffu, g, o);
-                }
-                if (g != T(0) && fabs((double)g) > thresh * sqrt((double)a * (double)b)) {
-                    const T zeta = (b - a) / (T(2) * g);
-                    const T tt = (zeta >= T(0) ? T(1) : T(-1)) / (fabs(zeta) + sqrt(T(1) + zeta * zeta));
-                    const T c = T(1) / sqrt(T(1) + tt * tt), sn = c * tt;
-                    T* zp = Z + (size_t)p * r;
-                    T* zq = Z + (size_t)q * r;
-                    for (int i = lane; i < r; i += 32) {
-                        const T x = mp[i], y = mq[i];
-                        mp[i] = c * x - sn * y;
-                        mq[i] = sn * x + c * y;
-                        const T u = zp[i], v = zq[i];
-                        zp[i] = c * u - sn * v;
-                        zq[i] = sn * u + c * v;
-                    }
-                    if (lane == 0) *s_rot = 1;
+                    const T x = mp[i], y = mq[i];
+                    mp[i] = c * x - sn * y;
+                    mq[i] = sn * x + c * y;
+                    const T u = zp[i], v = zq[i];
+                    zp[i] = c * u - sn * v;
+                    zq[i] = sn * u + c * v;
                 }
             }
             __syncthreads();
         }
-        const int rot = *s_rot;
-        __syncthreads();
-        if (!rot) break;
+        if (!rotated) break;
     }
 }
 
@@ -456,12 +560,15 @@ __global__ void __launch_bounds__(ACA_NT) k_recompress(const RecJob* __restrict_
     double* sig = cbuf + (J0R + 3);   // R + 3
     int* idx = reinterpret_cast<int*>(sig + (J0R + 3));
     __shared__ double sv[ACA_NW];
-    __shared__ int s_rot;
+    __shared__ union {
+        JacobiRound<float> f;
+        JacobiRound<double> d;
+    } s_jac;
     const RecJob J = jobs[blockIdx.x];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int r = J.r;
     if (r == 0) {
-        if (tid == 0) rank_out[blockIdx.x] = 0;
+        if (tid == 0) rank_out[J.id] = 0;
         return;
     }
     double* U = ws + J.ws_off;
@@ -491,13 +598,14 @@ __global__ void __launch_bounds__(ACA_NT) k_recompress(const RecJob* __restrict_
     float* Zf = Mf + (size_t)r * r;
     double f2 = 0.0;
     for (int q = tid; q < r * r; q += ACA_NT) f2 += M[q] * M[q];
-    const double fn = sqrt(block_sum(f2, sv));  // rotations do not see the scale: M / ||M||_F in FP32
+    const double fn = sqrt(block_sum<ACA_NW>(f2, sv));  // rotations do not see the scale: M / ||M||_F in FP32
     for (int q = tid; q < r * r; q += ACA_NT) {
         Mf[q] = fn > 0.0 ? (float)(M[q] / fn) : 0.f;
         Zf[q] = (q % r == q / r) ? 1.f : 0.f;
     }
     __syncthreads();
-    jacobi_sweeps<float>(Mf, Zf, r, 1e-5, 15, &s_rot);
+    jacobi_sweeps<float>(Mf, Zf, r, 1e-5, 15, s_jac.f);
+    __syncthreads();
     int bad = 0;
     for (int q = tid; q < r * r; q += ACA_NT) bad |= !isfinite(Zf[q]);
     bad = __syncthreads_or(bad);
@@ -514,7 +622,8 @@ __global__ void __launch_bounds__(ACA_NT) k_recompress(const RecJob* __restrict_
     __syncthreads();
     for (int q = tid; q < r * r; q += ACA_NT) M[q] = RV[q];
     __syncthreads();
-    jacobi_sweeps<double>(M, Z, r, 1e-15, 30, &s_rot);
+    jacobi_sweeps<double>(M, Z, r, 1e-15, 30, s_jac.d);
+    __syncthreads();
     // singular values, order by decreasing value, truncation rank
     for (int j = w; j < r; j += ACA_NW) {
         double a = 0.0;
@@ -542,7 +651,7 @@ __global__ void __launch_bounds__(ACA_NT) k_recompress(const RecJob* __restrict_
             --k;
         }
         for (int j = 0; j < r; ++j) ord[j] = (double)idx[j];
-        rank_out[blockIdx.x] = k;
+        rank_out[J.id] = k;
     }
 }
 
@@ -576,7 +685,7 @@ void launch_aca(const ElemRec* el, const AcaJob* jobs, int njobs, int max_sn, do
     if (smem > 200 * 1024) fail(HM_EINVAL, "assemble: cluster too large for the ACA kernel");
     if (smem > 48 * 1024)
         HM_CUDA(cudaFuncSetAttribute(k_aca, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_aca<<<(unsigned)njobs, ACA_NT, smem, st>>>(el, jobs, ws, R, eps, mu, nu, rank_out, status_out, evals);
+    k_aca<<<(unsigned)njobs, CROSS_NT, smem, st>>>(el, jobs, ws, R, eps, mu, nu, rank_out, status_out, evals);
     HM_LAUNCH_CHECK();
 }
 

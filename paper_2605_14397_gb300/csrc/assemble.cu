@@ -218,6 +218,7 @@ void assemble(const Tree& T, const hm_assemble_opts& opt, cudaStream_t st, HMat&
             J.s_n = F.s_n;
             J.t_begin = F.t_begin;
             J.t_n = F.t_n;
+            J.id = (int32_t)jobs.size();
             J.ws_off = wlen;
             jobs.push_back(J);
             wlen += need;
@@ -227,7 +228,14 @@ void assemble(const Tree& T, const hm_assemble_opts& opt, cudaStream_t st, HMat&
         const int64_t nb = b1 - b0;
         if ((size_t)wlen > ws.n) ws.alloc(wlen);
         DevBuf<AcaJob> d_jobs;
-        d_jobs.upload(jobs, st);
+        {
+            // largest blocks first: a CTA per block, and the last ones to start should be short
+            std::vector<AcaJob> sorted(jobs);
+            std::stable_sort(sorted.begin(), sorted.end(), [](const AcaJob& x, const AcaJob& y) {
+                return x.s_n + x.t_n > y.s_n + y.t_n;
+            });
+            d_jobs.upload(sorted, st);
+        }
         if ((int64_t)d_rank.n < nb) { d_rank.alloc(nb); d_stat.alloc(nb); }
         launch_aca(H.elems.p, d_jobs.p, (int)nb, max_sn, ws.p, R, eps_aca, mu, opt.nu, d_rank.p, d_stat.p,
                    d_evals.p, st);
@@ -269,6 +277,7 @@ void assemble(const Tree& T, const hm_assemble_opts& opt, cudaStream_t st, HMat&
             J.mT = 3 * F.t_n;
             J.r = ranks[b];
             J.R = R;
+            J.id = (int32_t)rj.size();
             rj.push_back(J);
             rj_block.push_back(b);
             slen += 5LL * J.r * J.r + J.r;  // R_U, R_V, M, Z, order, FP32 copies of M and Z
@@ -277,7 +286,11 @@ void assemble(const Tree& T, const hm_assemble_opts& opt, cudaStream_t st, HMat&
         if (!rj.empty()) {
             if ((size_t)slen > small.n) small.alloc(std::max<int64_t>(slen, 1));
             DevBuf<RecJob> d_rj;
-            d_rj.upload(rj, st);
+            std::vector<RecJob> sorted(rj);
+            auto cost = [](const RecJob& x) { return ((int64_t)x.mS + x.mT + 8 * x.r) * x.r * x.r; };
+            std::stable_sort(sorted.begin(), sorted.end(),
+                             [&](const RecJob& x, const RecJob& y) { return cost(x) > cost(y); });
+            d_rj.upload(sorted, st);
             launch_recompress(d_rj.p, (int)rj.size(), R, ws.p, small.p, tau, d_rank.p, st);
             HM_CUDA(cudaMemcpyAsync(krank.data(), d_rank.p, rj.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
             HM_CUDA(cudaStreamSynchronize(st));
