@@ -108,15 +108,15 @@ __device__ __forceinline__ void acc_fma2(float& a0, float& a1, float v, Z32 z0, 
     a0 = r.x;
     a1 = r.y;
 }
-// the RHS of one coefficient: pairs for FP32 accumulators, one by one otherwise
-template <int NR, class A, class Z>
-__device__ __forceinline__ void acc_fma_rhs(A* acc, float v, const Z* z, int stride) {
-    if constexpr (std::is_same<A, float>::value && NR % 2 == 0) {
+// the operands of one column for NR right-hand sides (a multiple of 4) as pairs (p: the
+// column's interleaved values in shared memory, 16-byte aligned)
+template <int NR>
+__device__ __forceinline__ void load_z2(float2 (&z)[NR / 2], const float* p) {
 #pragma unroll
-        for (int k = 0; k < NR; k += 2) acc_fma2(acc[k * stride], acc[(k + 1) * stride], v, z[k], z[k + 1]);
-    } else {
-#pragma unroll
-        for (int k = 0; k < NR; ++k) acc_fma(acc[k * stride], v, z[k]);
+    for (int q = 0; q < NR / 4; ++q) {
+        const float4 f = reinterpret_cast<const float4*>(p)[q];
+        z[2 * q] = make_float2(f.x, f.y);
+        z[2 * q + 1] = make_float2(f.z, f.w);
     }
 }
 // one step of the compensated dot product: acc += a (zh + zl)
@@ -188,27 +188,6 @@ __device__ __forceinline__ double part_value(float2 a) { return (double)a.x + (d
 template <class Part>
 using PartSum = decltype(part_value(Part()));
 
-// z operands of one column for NR right-hand sides (p: the column's nr interleaved
-// values in shared memory).  With nr == NR (a multiple of 4 for floats, of 2 for
-// doubles) the values are 16-byte aligned and read as vectors.
-template <int NR>
-__device__ __forceinline__ void load_z(Z32 (&z)[NR], const float* p, int nr) {
-    if constexpr (NR % 4 == 0) {
-        if (nr == NR) {
-#pragma unroll
-            for (int q = 0; q < NR / 4; ++q) {
-                const float4 f = reinterpret_cast<const float4*>(p)[q];
-                z[4 * q] = Z32{f.x};
-                z[4 * q + 1] = Z32{f.y};
-                z[4 * q + 2] = Z32{f.z};
-                z[4 * q + 3] = Z32{f.w};
-            }
-            return;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < NR; ++k) z[k] = make_z(k < nr ? p[k] : 0.f);
-}
 // the (hi, lo) operands of one column for NR right-hand sides in F64 mode (16-byte aligned
 // for an even NR)
 template <int NR>
@@ -265,17 +244,25 @@ __device__ __forceinline__ float bf16_value(uint32_t b) { return __uint_as_float
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// xc[dof * nr + k] = x[k * ndof + user dof]
-template <class V>
-__global__ void k_gather(const V* __restrict__ x, V* __restrict__ xc, const int32_t* __restrict__ perm, int64_t N,
-                         int nrhs) {
+// xc[dof * np + k] = x[k * ndof + user dof], zero for k >= nrhs (np: the padded count)
+__global__ void k_gather(const float* __restrict__ x, float* __restrict__ xc, const int32_t* __restrict__ perm,
+                         int64_t N, int nrhs, int np) {
     pdl_trigger();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t ndof = 3 * N;
-    if (q >= ndof * nrhs) return;
-    const int64_t r = q / nrhs, k = q % nrhs;
+    if (q >= ndof * np) return;
+    const int64_t r = q / np, k = q % np;
     const int64_t p = r / 3, m = r % 3;
-    xc[q] = x[k * ndof + 3 * (int64_t)perm[p] + m];
+    xc[q] = k < nrhs ? x[k * ndof + 3 * (int64_t)perm[p] + m] : 0.f;
+}
+
+// the same padding for operands already in cluster order, interleaved by nr
+__global__ void k_pad(const float* __restrict__ xc, float* __restrict__ xp, int64_t ndof, int nr, int np) {
+    pdl_trigger();
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q >= ndof * np) return;
+    const int64_t r = q / np, k = q % np;
+    xp[q] = k < nr ? xc[r * nr + k] : 0.f;
 }
 
 // F64 gather: xc[dof * nr + k] = (hi, lo) split of x[k * ndof + user dof]
@@ -659,7 +646,7 @@ struct StreamArgs {
     int32_t* counters;
     int* err;
     int64_t ndof;
-    int nr;       // right-hand sides in this launch (<= NR); also the interleave stride
+    int nout;     // right-hand sides the caller asked for (the vectors of out); the rest pad the kernel's count
     int ld_max;
     const int* skip;  // optional device flag: when set, the kernels return at once
     uint64_t wait_ns; // limit of every bounded wait of the copy ring
@@ -729,9 +716,9 @@ __device__ __forceinline__ void produce(const StreamArgs& a, unsigned char* smem
         }
         if constexpr (WITH_Z) {
             const V* zsrc = (const V*)(ch.kind == 0 ? a.xc : a.tb);
-            const int64_t z0 = ch.zoff * a.nr;
+            const int64_t z0 = ch.zoff * NR;
             const int64_t a0 = z0 & ~(int64_t)(ZR::ALIGN - 1);
-            const int64_t a1 = (z0 + (int64_t)ch.ncols * a.nr + ZR::ALIGN - 1) & ~(int64_t)(ZR::ALIGN - 1);
+            const int64_t a1 = (z0 + (int64_t)ch.ncols * NR + ZR::ALIGN - 1) & ~(int64_t)(ZR::ALIGN - 1);
             const uint32_t zbytes = (uint32_t)((a1 - a0) * (int64_t)sizeof(V));
             mbar_arrive_expect_tx(full + s, bytes + zbytes);
             bulk_g2s(stg, zsrc + a0, zbytes, full + s);
@@ -803,6 +790,56 @@ __device__ __forceinline__ void ff_columns_n(FF (&t)[NR][RPW], int nact, const E
         ff_columns<2>(t, col0, ld, zb, c0, ncols, step);
 }
 
+// Several right-hand sides in F32 mode: columns c0, c0 + step, ... of a chunk against the NA
+// row blocks of 32 rows this warp holds, accumulators in RHS pairs for the packed FMA.  The
+// row block count is a template argument and the right-hand sides are NR exactly (the host
+// pads their number), so a column is its loads and FMAs only (with both tested in the loop a
+// column of three blocks and 16 RHS took 62 instructions, 24 of them FMAs).  16 RHS on three
+// 100 x 100 planes (1.92 GB, 282 us at the copy bandwidth): 540 us before, 395 now.
+template <int NA, int NR, int RPW, class E>
+__device__ __forceinline__ void mr_columns(float2 (&t)[RPW][NR / 2], const E* col0, int ld, const float* zb, int c0,
+                                           int ncols, int step) {
+    const E* col = col0 + (size_t)c0 * ld;
+    const float* zc = zb + (size_t)c0 * NR;
+    const int cs = step * ld, zs = step * NR;
+    for (int c = c0; c < ncols; c += step, col += cs, zc += zs) {
+        float v[NA];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) v[i] = coef(col, 32 * i);
+        float2 z[NR / 2];
+        load_z2<NR>(z, zc);
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            const float2 vv = make_float2(v[i], v[i]);
+#pragma unroll
+            for (int k = 0; k < NR / 2; ++k) t[i][k] = __ffma2_rn(vv, z[k], t[i][k]);
+        }
+    }
+}
+// the same for a run-time row block count (0 .. RPW)
+template <int NR, int RPW, class E>
+__device__ __forceinline__ void mr_columns_n(float2 (&t)[RPW][NR / 2], int nact, const E* col0, int ld,
+                                             const float* zb, int c0, int ncols, int step) {
+    static_assert(RPW == 2 || RPW == 3 || RPW == 6, "one variant per row block count");
+    if constexpr (RPW <= 3) {
+        if (RPW == 3 && nact == 3)
+            mr_columns<RPW, NR>(t, col0, ld, zb, c0, ncols, step);
+        else if (nact == 2)
+            mr_columns<2, NR>(t, col0, ld, zb, c0, ncols, step);
+        else if (nact == 1)
+            mr_columns<1, NR>(t, col0, ld, zb, c0, ncols, step);
+    } else {
+        if (nact == 6)
+            mr_columns<6, NR>(t, col0, ld, zb, c0, ncols, step);
+        else if (nact == 5)
+            mr_columns<5, NR>(t, col0, ld, zb, c0, ncols, step);
+        else if (nact >= 3)
+            mr_columns<4, NR>(t, col0, ld, zb, c0, ncols, step);
+        else if (nact >= 1)
+            mr_columns<2, NR>(t, col0, ld, zb, c0, ncols, step);
+    }
+}
+
 // ---- phase 2: y = [D | U] z per row leaf
 // RS > 1 splits each column's rows over RS warps (RPL / RS rows per lane each), so that
 // many right-hand sides fit in registers with more warps in flight.
@@ -817,14 +854,14 @@ template <int MODE, class C, int NR, int RPL, int NCW, int RS, int ST = STAGES>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     constexpr bool TC2 = MODE == 0 && NR == 1 && RS == 1 && NCW == 16 && RPL == 6 &&
                          std::is_same<C, uint16_t>::value;
-    // BF16 U slices with 16 RHS (TC16, when the launch has exactly 16): warp w < 12 owns
-    // m-tile w (rows 16 w .. 16 w + 15 of the leaf) and both n-tiles (RHS 0-7, 8-15); A as
+    // BF16 U slices with 16 RHS (TC16): warp w owns the m-tiles w / 2 and w / 2 + 8 (16 rows
+    // of the leaf each) of the n-tile w % 2 (8 RHS); A as
     // in TC2, B = t in the packed BF16 (hi, lo) form of k_reduce_pack16_mix read with
-    // ldmatrix.trans, two mma per n-tile and k-tile.  The CUDA-core accumulators keep the
+    // ldmatrix.trans, two mma per k-tile in two chains.  The CUDA-core accumulators keep the
     // near tiles; the tensor-core results join them at the flush through ty.
-    constexpr bool TC16 = MODE == 0 && NR == 16 && RS == 2 && NCW == 16 && RPL == 6 &&
+    constexpr bool TC16 = MODE == 0 && NR == 16 && RS == 2 && NCW == 16 && RPL <= 6 &&
                           std::is_same<C, uint16_t>::value;
-    constexpr int TC16_MT = 12, TY_LD = 196;  // m-tiles (192 rows); ty row stride (bank spread)
+    constexpr int TC16_MT = 2 * RPL, TY_LD = 196;  // m-tiles of 16 rows; ty row stride (bank spread)
     constexpr int TKG = 4, TMG = 4, TMT = 3;  // k-groups x m-groups = NCW; m-tiles per warp
     static_assert(!TC2 || (TKG * TMG == NCW && TMG * TMT * 16 >= 32 * RPL && TKG * 2 * 16 >= MAX_CHUNK_COLS),
                   "tensor-core phase 2 covers every row and column");
@@ -845,7 +882,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     // FP32 vectors with 16 RHS on leaves of up to 64 elements reduce 8 RHS per pass of the
     // flush (4 barriers per leaf instead of 32); the other variants one RHS per pass (their
     // reduction buffer would not fit beside the ring)
-    constexpr int KP = (MODE == 0 && NR == 16 && RPL == 6) ? 8 : 1;
+    constexpr int KP = (MODE == 0 && NR == 16 && RPL <= 6) ? 8 : 1;
     Acc* red = (Acc*)(stage + (size_t)ST * STRIDE);  // [KP][NG][32 RPL]
     float* ty = (float*)(red + (size_t)KP * NG * 32 * RPL);  // TC16: the leaf's tensor-core sums [16 RHS][TY_LD]
 
@@ -864,9 +901,10 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     Vv* yc = (Vv*)a.out;
     Vv* slots = (Vv*)a.slots;
     const int g = w / RS, rbase = (w % RS) * 32 * RPW;
-    Acc acc[NR][RPW];
+    constexpr bool MR = MODE == 0 && NR > 1;  // accumulators in RHS pairs
+    Acc acc[MR ? 1 : NR][RPW];
+    float2 acc2[MR ? RPW : 1][MR ? NR / 2 : 1];
     float dt[TMT][4];  // TC2: this warp's m-tiles of the leaf (tensor-core part)
-    const bool tc16 = TC16 && a.nr == 16;
     int cur = -1, rot = 0;
     LeafDesc L{};
 
@@ -879,12 +917,17 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
         // runtime index into acc would move it to local memory)
 #pragma unroll
         for (int k0 = 0; k0 < NR; k0 += KP) {
-            if (k0 >= a.nr) break;
+            if (k0 >= a.nout) break;
 #pragma unroll
             for (int kk = 0; kk < KP; ++kk)
 #pragma unroll
-                for (int i = 0; i < RPW; ++i)
-                    red[((size_t)kk * NG + g) * (32 * RPL) + rbase + lane + 32 * i] = acc[k0 + kk][i];
+                for (int i = 0; i < RPW; ++i) {
+                    Acc& o = red[((size_t)kk * NG + g) * (32 * RPL) + rbase + lane + 32 * i];
+                    if constexpr (MR)
+                        o = ((k0 + kk) & 1) ? acc2[i][(k0 + kk) / 2].y : acc2[i][(k0 + kk) / 2].x;
+                    else
+                        o = acc[k0 + kk][i];
+                }
             if constexpr (TC2) {
                 // lanes 4 c hold rows 16 mt + c (d0 + d1) and 16 mt + c + 8 (d2 + d3)
                 __syncwarp();
@@ -900,13 +943,11 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
             consumer_sync(NCW * 32);
             for (int e = threadIdx.x; e < KP * rows; e += NCW * 32) {
                 const int kk = e / rows, r = e - kk * rows, k = k0 + kk;
-                if (k >= a.nr) continue;
+                if (k >= a.nout) continue;
                 const Acc* rk = red + (size_t)kk * NG * (32 * RPL);
                 Acc s = rk[r];
                 for (int q = 1; q < NG; ++q) acc_add(s, rk[(size_t)q * (32 * RPL) + r]);
-                if constexpr (TC16) {
-                    if (tc16) acc_add(s, ty[(size_t)k * TY_LD + r]);
-                }
+                if constexpr (TC16) acc_add(s, ty[(size_t)k * TY_LD + r]);
                 if (whole)
                     yc[(int64_t)k * a.ndof + 3 * (int64_t)L.begin + r] = (Vv)acc_value(s);
                 else
@@ -924,7 +965,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
             consumer_sync(NCW * 32);
             if (*s_flag) {
                 __threadfence();
-                for (int k = 0; k < a.nr; ++k)
+                for (int k = 0; k < a.nout; ++k)
                     for (int r = threadIdx.x; r < rows; r += NCW * 32) {
                         Vv s = 0;
                         for (int p = 0; p < sp.nparts; ++p)
@@ -946,73 +987,71 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
             if (cur >= 0) flush();
             cur = ch.leaf;
             L = a.leaves[cur];
+            if constexpr (MR) {
 #pragma unroll
-            for (int k = 0; k < NR; ++k)
+                for (int j = 0; j < RPW; ++j)
 #pragma unroll
-                for (int j = 0; j < RPW; ++j) acc_zero(acc[k][j]);
+                    for (int k = 0; k < NR / 2; ++k) acc2[j][k] = make_float2(0.f, 0.f);
+            } else {
+#pragma unroll
+                for (int k = 0; k < NR; ++k)
+#pragma unroll
+                    for (int j = 0; j < RPW; ++j) acc_zero(acc[k][j]);
+            }
 #pragma unroll
             for (int j = 0; j < TMT; ++j) dt[j][0] = dt[j][1] = dt[j][2] = dt[j][3] = 0.f;
             if constexpr (TC16) {
-                // the entries of ty this lane accumulates (its m-tile, see below) start at 0
-                if (tc16 && w < TC16_MT) {
-                    const int r0 = 16 * w + (lane >> 2), c0 = 2 * (lane & 3);
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) {
-                        float* col = ty + (size_t)(8 * nt + c0) * TY_LD;
-                        col[r0] = col[TY_LD + r0] = col[r0 + 8] = col[TY_LD + r0 + 8] = 0.f;
-                    }
+                // the entries of ty this lane accumulates (its m-tiles, see below) start at 0
+                for (int mt = w >> 1; mt < TC16_MT; mt += 8) {
+                    const int r0 = 16 * mt + (lane >> 2);
+                    float* col = ty + (size_t)(8 * (w & 1) + 2 * (lane & 3)) * TY_LD;
+                    col[r0] = col[TY_LD + r0] = col[r0 + 8] = col[TY_LD + r0 + 8] = 0.f;
                 }
             }
         }
         mbar_wait(full + s, (uint32_t)(q / ST) & 1u, a.err, 1, a.wait_ns);
         const unsigned char* stg = stage + (size_t)s * STRIDE;
-        const int64_t z0 = ch.zoff * a.nr;
+        const int64_t z0 = ch.zoff * NR;
         using Zin = typename AccT<MODE>::zin;  // same size as Vv
         const Zin* zb = (const Zin*)stg + (z0 - (z0 & ~(int64_t)(ZR::ALIGN - 1)));
         const unsigned char* buf = stg + ZR::BYTES;
         const int rows = 3 * L.n;
         const int cg = deal_start<NG>(g, rot);  // this warp's first column on the CUDA cores
         if constexpr (TC16) {
-            if (tc16 && ch.kind != 0) {
-                if (w < TC16_MT && 16 * w < rows) {
-                    float d16[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-                    const uint16_t* ub = (const uint16_t*)buf;
-                    const int ld = ch.ld, ncols = ch.ncols;
-                    const int j8 = lane >> 3, i8 = lane & 7;
-                    const int m0 = 16 * w + (j8 & 1) * 8;
-                    const uint32_t zaddr = smem_u32(zline);
-                    const uint32_t tbase = smem_u32(stg);  // packed t of the chunk: 64 B per column
-                    for (int kt = 0; kt * 16 < ncols; ++kt) {
-                        // A: this lane addresses slice column kt 16 + (j8 / 2) 8 + i8, rows m0 ..
-                        const int kc = kt * 16 + (j8 >> 1) * 8 + i8;
-                        const uint32_t aaddr = (kc < ncols && m0 < ld) ? smem_u32(ub + (size_t)kc * ld + m0) : zaddr;
-                        uint32_t a0, a1, a2, a3;
+            if (ch.kind != 0) {
+                const uint16_t* ub = (const uint16_t*)buf;
+                const int ld = ch.ld, ncols = ch.ncols;
+                const int j8 = lane >> 3, i8 = lane & 7, nt = w & 1;
+                const uint32_t zaddr = smem_u32(zline);
+                // B: matrix j8 = (k half j8 % 2, BF16 high or low part j8 / 2), row i8 = column
+                // kb of t in the packed form (64 bytes a column)
+                const uint32_t tbase = smem_u32(stg) + 64u * (uint32_t)((j8 & 1) * 8 + i8);
+                const int lg0 = (int)(ch.zoff & 7) + (j8 & 1) * 8 + i8, piece = 2 * nt + (j8 >> 1);
+                for (int mt = w >> 1; 16 * mt < rows; mt += 8) {
+                    const int m0 = 16 * mt + (j8 & 1) * 8;
+                    const uint32_t abase = smem_u32(ub + m0);
+                    float dh[4] = {0.f, 0.f, 0.f, 0.f}, dl[4] = {0.f, 0.f, 0.f, 0.f};
+                    for (int k0 = 0; k0 < ncols; k0 += 16) {
+                        // A: this lane addresses slice column k0 + (j8 / 2) 8 + i8, rows m0 ..
+                        const int kc = k0 + (j8 >> 1) * 8 + i8, kb = k0 + (j8 & 1) * 8 + i8;
+                        const uint32_t aaddr = kc < ncols && m0 < ld ? abase + 2u * (uint32_t)(kc * ld) : zaddr;
+                        const uint32_t badd =
+                            kb < ncols ? tbase + 64u * (uint32_t)k0 + 16u * (uint32_t)tb16_piece_pos(lg0 + k0, piece)
+                                       : zaddr;
+                        uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
                         ldsm_x4_t(aaddr, a0, a1, a2, a3);
-                        // B: matrix j8 = (k half j8 % 2, n-tile j8 / 2), row i8 = column kb of t
-                        const int kb = kt * 16 + (j8 & 1) * 8 + i8;
-                        const int64_t lg = ch.zoff + kb;
-                        const uint32_t rowaddr = tbase + 64u * (uint32_t)kb;
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {  // BF16 high parts of t, then the low parts
-                            const uint32_t badd =
-                                kb < ncols ? rowaddr + 16u * (uint32_t)tb16_piece_pos(lg, 2 * (j8 >> 1) + h) : zaddr;
-                            uint32_t b0, b1, b2, b3;
-                            ldsm_x4_t(badd, b0, b1, b2, b3);
-                            mma_bf16(d16[0], a0, a1, a2, a3, b0, b1);
-                            mma_bf16(d16[1], a0, a1, a2, a3, b2, b3);
-                        }
+                        ldsm_x4_t(badd, b0, b1, b2, b3);
+                        mma_bf16(dh, a0, a1, a2, a3, b0, b1);  // BF16 high parts of t
+                        mma_bf16(dl, a0, a1, a2, a3, b2, b3);  // the low parts
                     }
-                    // d16: rows 16 w + lane / 4 (c0, c1) and + 8 (c2, c3), RHS 8 nt + 2 (lane % 4)
-                    // + {0, 1}; summed over the leaf's chunks in ty, read by the flush
-                    const int r0 = 16 * w + (lane >> 2), c0 = 2 * (lane & 3);
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) {
-                        float* col = ty + (size_t)(8 * nt + c0) * TY_LD;
-                        col[r0] += d16[nt][0];
-                        col[TY_LD + r0] += d16[nt][1];
-                        col[r0 + 8] += d16[nt][2];
-                        col[TY_LD + r0 + 8] += d16[nt][3];
-                    }
+                    // rows 16 mt + lane / 4 (c0, c1) and + 8 (c2, c3), RHS 8 nt + 2 (lane % 4) +
+                    // {0, 1}; summed over the leaf's chunks in ty, read by the flush
+                    const int r0 = 16 * mt + (lane >> 2);
+                    float* col = ty + (size_t)(8 * nt + 2 * (lane & 3)) * TY_LD;
+                    col[r0] += dh[0] + dl[0];
+                    col[TY_LD + r0] += dh[1] + dl[1];
+                    col[r0 + 8] += dh[2] + dl[2];
+                    col[TY_LD + r0 + 8] += dh[3] + dl[3];
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty + s);
@@ -1060,53 +1099,43 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
         // Rows at or beyond `rows` read whatever follows the column in shared memory (the
         // next column, stage or the reduction buffer: always inside the allocation); their
         // accumulators are never flushed, so no bound check is needed per coefficient.
-        // With several RHS a warp skips its row blocks past the leaf (leaves of fewer than
-        // 64 elements), a warp-uniform test; with one RHS the loop stays branch-free.
-        if constexpr (MODE == 1) {
-            const int nact = max(0, min(RPW, (rows - rbase + 31) >> 5));
-            rot = deal_next<NG>(rot, ch.ncols);
-            if (ch.kind == 0)
-                ff_columns_n(acc, nact, (const float*)buf + rbase + lane, ch.ld, zb, cg, ch.ncols, NG);
-            else
-                ff_columns_n(acc, nact, (const C*)buf + rbase + lane, ch.ld, zb, cg, ch.ncols, NG);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(empty + s);
-            continue;
-        } else {
-        const int nact = NR == 1 ? RPW : max(0, min(RPW, (rows - rbase + 31) >> 5));
+        // Except in the HBM-bound single-RHS F32 loop a warp skips the row blocks past the
+        // leaf.
         rot = deal_next<NG>(rot, ch.ncols);
-        for (int c = cg; c < ch.ncols && nact > 0; c += NG) {
-            Z32 zv[NR];
-            if constexpr (NR == 1)
-                zv[0] = make_z(zb[c]);
+        const int nact = max(0, min(RPW, (rows - rbase + 31) >> 5));
+        const float* near_col = (const float*)buf + rbase + lane;
+        const C* u_col = (const C*)buf + rbase + lane;
+        if constexpr (MODE == 1) {
+            if (ch.kind == 0)
+                ff_columns_n(acc, nact, near_col, ch.ld, zb, cg, ch.ncols, NG);
             else
-                load_z<NR>(zv, zb + (size_t)c * a.nr, a.nr);
-            if (ch.kind == 0) {
-                const float* col = (const float*)buf + (size_t)c * ch.ld + rbase + lane;
+                ff_columns_n(acc, nact, u_col, ch.ld, zb, cg, ch.ncols, NG);
+        } else if constexpr (MR) {
+            if (ch.kind == 0)
+                mr_columns_n<NR>(acc2, nact, near_col, ch.ld, zb, cg, ch.ncols, NG);
+            else
+                mr_columns_n<NR>(acc2, nact, u_col, ch.ld, zb, cg, ch.ncols, NG);
+        } else {
+            for (int c = cg; c < ch.ncols; c += NG) {
+                const Z32 zv = make_z(zb[c]);
+                if (ch.kind == 0) {
+                    const float* col = near_col + (size_t)c * ch.ld;
 #pragma unroll
-                for (int ii = 0; ii < RPW; ++ii) {
-                    if (NR > 1 && ii >= nact) break;
-                    const float v = col[32 * ii];
-                    acc_fma_rhs<NR>(&acc[0][ii], v, zv, RPW);
-                }
-            } else {
-                const C* col = (const C*)buf + (size_t)c * ch.ld + rbase + lane;
+                    for (int ii = 0; ii < RPW; ++ii) acc_fma(acc[0][ii], col[32 * ii], zv);
+                } else {
+                    const C* col = u_col + (size_t)c * ch.ld;
 #pragma unroll
-                for (int ii = 0; ii < RPW; ++ii) {
-                    if (NR > 1 && ii >= nact) break;
-                    const float v = coef(col, 32 * ii);
-                    acc_fma_rhs<NR>(&acc[0][ii], v, zv, RPW);
+                    for (int ii = 0; ii < RPW; ++ii) acc_fma(acc[0][ii], coef(col, 32 * ii), zv);
                 }
             }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(empty + s);
-        }
     }
     if (cur >= 0) flush();
 }
 
-// ---- phase 1: P = V_t^T xc_t, one partial per V column (F32 mode)
+// ---- phase 1: P = V_t^T xc_t, one partial per V column (F32 mode, 1 to 4 right-hand sides)
 template <class C, int NR, int RPL, int NCW, int ST = STAGES>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
     using Acc = float;
@@ -1159,7 +1188,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
                 const int r = PAIR ? 2 * lane + 64 * (ii >> 1) + (ii & 1) : lane + 32 * ii;
 #pragma unroll
                 for (int k = 0; k < NR; ++k)
-                    xr[k][ii] = make_z((r < rows && k < a.nr) ? xs[(3 * (int64_t)L.begin + r) * a.nr + k] : 0.f);
+                    xr[k][ii] = make_z(r < rows ? xs[(3 * (int64_t)L.begin + r) * NR + k] : 0.f);
             }
         }
         mbar_wait(full + s, (uint32_t)(q / ST) & 1u, a.err, 1, a.wait_ns);
@@ -1226,8 +1255,161 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
                 }
             }
             const int k = warp_reduce_scatter<NR>(acc, lane);
-            if ((lane & (32 / NR - 1)) == 0 && k < a.nr) P[(ch.zoff + c) * a.nr + k] = (Vv)acc_value(acc[0]);
+            if ((lane & (32 / NR - 1)) == 0) P[(ch.zoff + c) * NR + k] = (Vv)acc_value(acc[0]);
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty + s);
+    }
+}
+
+// ---- phase 1 with 5 to 16 right-hand sides (F32 mode)
+//
+// A warp takes 4 CL neighbouring columns: lane (cg, rl) = (lane / 8, lane % 8) columns
+// cg + 4 j (j < CL) and the four rows 4 rl .. 4 rl + 3 of every 32, so that the sums over
+// rows meet over 8 lanes only -- 28 shuffles for 8 columns of 16 RHS, where lanes over the
+// rows of one column at a time took 16 a column and as many instructions to reduce as to
+// multiply (155 a column in all; now about 85).  Coefficients come as 16-byte reads of a
+// column (eight lanes read 128 bytes in a row), the leaf's operands from shared memory,
+// where they lie so that the eight lanes' 16-byte reads of one row and four RHS are
+// contiguous and the four column groups share them; every operand read serves CL columns.
+// x past the leaf's rows is zero, and everything an unchecked read can reach is
+// finite (the ring is zeroed first), so nothing is bound-checked.  Columns are dealt in units
+// of 4 CL across chunks; the ring is six deep because the warps work on about three chunks
+// at a time.  16 RHS take eight warps: 64 accumulators and their operands a lane.  Bound by the FP32 pipe and shared-memory reads: 16 RHS on three 100 x 100 planes
+// (0.82 GB of V, 0.12 ms at the copy bandwidth): 0.38 ms a column at a time, 0.21 ms now.
+template <class C>
+__device__ __forceinline__ float4 coef4(const C* p);
+template <>
+__device__ __forceinline__ float4 coef4<float>(const float* p) {
+    return *reinterpret_cast<const float4*>(p);
+}
+template <>
+__device__ __forceinline__ float4 coef4<uint16_t>(const uint16_t* p) {
+    const uint2 u = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xffff0000u));
+}
+
+constexpr int MR_STAGES = 6;
+// shared-memory float4 index of rows r (of 32 t + 4 rl + i), RHS 4 kq .. 4 kq + 3
+template <int NR>
+__device__ __forceinline__ int mr_x_index(int t, int i, int kq, int rl) {
+    return ((t * 4 + i) * (NR / 4) + kq) * 8 + rl;
+}
+
+template <class C, int NR, int NCW>
+__global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_mr(StreamArgs a) {
+    constexpr int CL = 4, UNIT = 4 * CL;  // columns of a lane, of a warp
+    constexpr int NV = CL * NR;           // accumulators of a lane
+    static_assert(NR == 8 || NR == 16, "after three halvings a lane holds NV / 8 sums of one column");
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t* full = (uint64_t*)smem;
+    uint64_t* empty = full + MR_STAGES;
+    unsigned char* stage = smem + BAR_BYTES;
+    float4* xs = (float4*)(stage + MR_STAGES * STAGE_BYTES + P1_TAIL);  // the leaf's operands (mr_x_index)
+    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, cg = lane >> 3, rl = lane & 7;
+    {
+        uint4* z = reinterpret_cast<uint4*>(stage);
+        for (int i = threadIdx.x; i < (MR_STAGES * STAGE_BYTES + P1_TAIL) / 16; i += blockDim.x)
+            z[i] = make_uint4(0u, 0u, 0u, 0u);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the copies write it
+    }
+    init_ring<MR_STAGES>(full, empty, NCW);
+    const int c0 = a.cta_begin[blockIdx.x], c1 = a.cta_begin[blockIdx.x + 1];
+    pdl_trigger();
+    if (w == NCW) {
+        // the V coefficients are constant: the copies start while the gather drains
+        if (lane == 0) produce<C, float, NR, false, false, MR_STAGES>(a, stage, STAGE_BYTES, full, empty, c0, c1);
+        return;
+    }
+    pdl_wait();  // x in cluster order comes from the preceding kernel
+    float* P = (float*)a.out;
+    const float* xg = (const float*)a.xc;
+    int cur = -1, nt = 0, rot = 0;
+    Chunk nxt = c0 < c1 ? a.chunks[c0] : Chunk{};
+    for (int i = c0; i < c1; ++i) {
+        const Chunk ch = nxt;
+        if (i + 1 < c1) nxt = a.chunks[i + 1];
+        const int q = i - c0, s = q % MR_STAGES;
+        if (ch.leaf != cur) {
+            consumer_sync(NCW * 32);  // every warp is past the leaf before
+            cur = ch.leaf;
+            const LeafDesc L = a.leaves[cur];
+            const int rows = 3 * L.n;
+            nt = (rows + 31) >> 5;
+            const float* xl = xg + 3 * (int64_t)L.begin * NR;
+            float* xf = reinterpret_cast<float*>(xs);
+            for (int e = threadIdx.x; e < nt * 32 * NR; e += NCW * 32) {
+                const int r = e / NR, k = e % NR;
+                const int at = mr_x_index<NR>(r >> 5, r & 3, k >> 2, (r & 31) >> 2);
+                xf[4 * at + (k & 3)] = r < rows ? xl[e] : 0.f;
+            }
+            consumer_sync(NCW * 32);
+        }
+        mbar_wait(full + s, (uint32_t)(q / MR_STAGES) & 1u, a.err, 1, a.wait_ns);
+        const C* buf = (const C*)(stage + (size_t)s * STAGE_BYTES);
+        const int units = (ch.ncols + UNIT - 1) / UNIT;
+        for (int u = deal_start<NCW>(w, rot); u < units; u += NCW) {
+            const C* colp[CL];
+#pragma unroll
+            for (int j = 0; j < CL; ++j)
+                colp[j] = buf + (size_t)min(u * UNIT + cg + 4 * j, ch.ncols - 1) * ch.ld + 4 * rl;
+            float2 acc[CL][NR / 2];
+#pragma unroll
+            for (int j = 0; j < CL; ++j)
+#pragma unroll
+                for (int k = 0; k < NR / 2; ++k) acc[j][k] = make_float2(0.f, 0.f);
+            for (int t = 0; t < nt; ++t) {
+                float v[CL][4];
+#pragma unroll
+                for (int j = 0; j < CL; ++j) {
+                    const float4 f = coef4<C>(colp[j] + 32 * t);
+                    v[j][0] = f.x, v[j][1] = f.y, v[j][2] = f.z, v[j][3] = f.w;
+                }
+#pragma unroll
+                for (int i4 = 0; i4 < 4; ++i4) {
+#pragma unroll
+                    for (int kq = 0; kq < NR / 4; ++kq) {
+                        const float4 x = xs[mr_x_index<NR>(t, i4, kq, rl)];
+#pragma unroll
+                        for (int j = 0; j < CL; ++j) {
+                            const float2 vv = make_float2(v[j][i4], v[j][i4]);
+                            acc[j][2 * kq] = __ffma2_rn(vv, make_float2(x.x, x.y), acc[j][2 * kq]);
+                            acc[j][2 * kq + 1] = __ffma2_rn(vv, make_float2(x.z, x.w), acc[j][2 * kq + 1]);
+                        }
+                    }
+                }
+            }
+            // NV sums over the 8 row lanes: halving exchanges leave each lane NV / 8 RHS of a column
+            float f[NV];
+#pragma unroll
+            for (int j = 0; j < CL; ++j)
+#pragma unroll
+                for (int k = 0; k < NR / 2; ++k) {
+                    f[j * NR + 2 * k] = acc[j][k].x;
+                    f[j * NR + 2 * k + 1] = acc[j][k].y;
+                }
+            int e = 0;
+#pragma unroll
+            for (int h = NV / 2, o = 4; o >= 1; h >>= 1, o >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int j = 0; j < h; ++j) {
+                    const float mine = up ? f[j + h] : f[j], other = up ? f[j] : f[j + h];
+                    f[j] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+                }
+                if (up) e += h;
+            }
+            const int c = u * UNIT + cg + 4 * (e / NR), k = e % NR;  // this lane: column c, RHS k ...
+            if (c < ch.ncols) {
+#pragma unroll
+                for (int j = 0; j < NV / 8; j += 4)
+                    *reinterpret_cast<float4*>(P + (ch.zoff + c) * NR + k + j) =
+                        make_float4(f[j], f[j + 1], f[j + 2], f[j + 3]);
+            }
+        }
+        rot = deal_next<NCW>(rot, units);
         __syncwarp();
         if (lane == 0) mbar_arrive(empty + s);
     }
@@ -1365,21 +1547,25 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_f64(StreamArgs a) 
 // shared memory, so ldmatrix reads A fragments directly), the B operand the leaf's rows
 // of x, each value split into BF16 hi + lo (two products, x kept to ~16 bits), kept in
 // registers for the whole leaf.  Warp w takes n-tile w % 2 (8 RHS) and m-tiles
-// w / 2, w / 2 + NCW / 2, ...; a lane whose ldmatrix row lies outside the chunk reads a
-// zeroed 16-byte line instead, so no access leaves the chunk.
+// w / 2, w / 2 + NCW / 2, ..., dealt across chunks; nothing is bound-checked: rows past the
+// leaf meet x = 0 and every byte a read can reach is finite (the ring is zeroed first).
 constexpr int TC_KT = 12;  // k-tiles of 16 rows: leaves of up to 192 rows
 
 template <int NCW>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_tc(StreamArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ __align__(16) uint16_t zline[8];
     uint64_t* full = (uint64_t*)smem;
     uint64_t* empty = full + STAGES;
     unsigned char* stage = smem + BAR_BYTES;
 
     if (a.skip && *(volatile const int*)a.skip) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x < 8) zline[threadIdx.x] = 0;
+    {  // finite data behind every unchecked read, as in k_phase1
+        uint4* z = reinterpret_cast<uint4*>(stage);
+        for (int i = threadIdx.x; i < (STAGES * STAGE_BYTES + P1_TAIL) / 16; i += blockDim.x)
+            z[i] = make_uint4(0u, 0u, 0u, 0u);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the copies write it
+    }
     init_ring(full, empty, NCW);
     const int c0 = a.cta_begin[blockIdx.x], c1 = a.cta_begin[blockIdx.x + 1];
     pdl_trigger();
@@ -1391,8 +1577,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_tc(StreamArgs a) {
     const float* xc = (const float*)a.xc;
     float* P = (float*)a.out;
     const int nt = w & 1;
-    const uint32_t zaddr = smem_u32(zline);
-    int cur = -1, rows = 0;
+    int cur = -1, rows = 0, rot = 0;
     uint32_t bh[TC_KT][2], bl[TC_KT][2];
     Chunk nxt = c0 < c1 ? a.chunks[c0] : Chunk{};
     for (int i = c0; i < c1; ++i) {
@@ -1429,26 +1614,29 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_tc(StreamArgs a) {
         const int ld = ch.ld, ncols = ch.ncols;
         const int mtiles = (ncols + 15) >> 4;
         const int j8 = lane >> 3, i8 = lane & 7;
-        for (int mt = w >> 1; mt < mtiles; mt += NCW / 2) {
-            const int m = mt * 16 + (j8 & 1) * 8 + i8;  // this lane's ldmatrix row (a V column)
-            float d[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int mt = deal_start<NCW / 2>(w >> 1, rot); mt < mtiles; mt += NCW / 2) {
+            // this lane's ldmatrix row: a V column; columns past the chunk repeat its last one
+            // and are not stored
+            const int m = min(mt * 16 + (j8 & 1) * 8 + i8, ncols - 1);
+            const uint32_t row = smem_u32(buf + (size_t)m * ld + (j8 >> 1) * 8);
+            float d[4] = {0.f, 0.f, 0.f, 0.f}, dl[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int kt = 0; kt < TC_KT; ++kt) {
-                const int k = kt * 16 + (j8 >> 1) * 8;
-                if (kt * 16 >= ld) break;
-                const uint32_t addr = (m < ncols && k < ld) ? smem_u32(buf + (size_t)m * ld + k) : zaddr;
+                if (kt * 16 >= rows) break;
                 uint32_t a0, a1, a2, a3;
-                ldsm_x4(addr, a0, a1, a2, a3);
+                ldsm_x4(row + 32u * kt, a0, a1, a2, a3);
                 mma_bf16(d, a0, a1, a2, a3, bh[kt][0], bh[kt][1]);
-                mma_bf16(d, a0, a1, a2, a3, bl[kt][0], bl[kt][1]);
+                mma_bf16(dl, a0, a1, a2, a3, bl[kt][0], bl[kt][1]);
             }
             // d0, d1: column mt*16 + lane/4, RHS nt*8 + 2 (lane % 4) + {0, 1}; d2, d3: column + 8
             const int col = mt * 16 + (lane >> 2), rhs = nt * 8 + 2 * (lane & 3);
             if (col < ncols)
-                *reinterpret_cast<float2*>(P + (ch.zoff + col) * 16 + rhs) = make_float2(d[0], d[1]);
+                *reinterpret_cast<float2*>(P + (ch.zoff + col) * 16 + rhs) = make_float2(d[0] + dl[0], d[1] + dl[1]);
             if (col + 8 < ncols)
-                *reinterpret_cast<float2*>(P + (ch.zoff + col + 8) * 16 + rhs) = make_float2(d[2], d[3]);
+                *reinterpret_cast<float2*>(P + (ch.zoff + col + 8) * 16 + rhs) =
+                    make_float2(d[2] + dl[2], d[3] + dl[3]);
         }
+        rot = deal_next<NCW / 2>(rot, mtiles);
         __syncwarp();
         if (lane == 0) mbar_arrive(empty + s);
     }
@@ -1497,11 +1685,11 @@ void mark(HMat& H, int idx, cudaStream_t st) {
 
 // consumer warps of phase 1 and phase 2, and phase 2's row split, per right-hand-side
 // count: as many warps as the per-thread registers (accumulators and operands) allow
-constexpr int ncw1_for(int NR) { return NR > 4 ? 8 : 16; }
-// F64 mode: six row blocks per warp whatever the leaf size
+// phase 2's row split: two or three row blocks per warp with 16 RHS, else (one F32 RHS apart)
+// six
 template <int MODE>
 constexpr int rs_for(int NR, int RPL) {
-    return MODE == 1 ? RPL / 6 : (NR > 4 ? 2 : 1);
+    return MODE == 0 && NR == 1 ? 1 : (NR == 16 ? (RPL == 4 ? 2 : RPL / 3) : RPL / 6);
 }
 
 // ST: ring depth; NCW1V / NCW2V: consumer warps of phase 1 / phase 2 (0: the default for
@@ -1517,21 +1705,27 @@ constexpr int ncw2_for(int NR, int RS) {
 
 template <int MODE, class C, int NR, int RPL, int ST = STAGES, int NCW1V = 0, int NCW2V = 0>
 void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool timed, cudaStream_t st) {
-    constexpr int NCW = NCW1V ? NCW1V : (MODE == 1 ? 16 : ncw1_for(NR)), RS = rs_for<MODE>(NR, RPL),
+    constexpr int NCW = NCW1V ? NCW1V : (MODE == 0 && NR == 16 ? 8 : 16), RS = rs_for<MODE>(NR, RPL),
                   NCW2 = NCW2V ? NCW2V : ncw2_for<MODE>(NR, RS);
     static_assert(MODE == 0 || (NR <= F64_PASS && ST == STAGES), "F64 passes");
     using Acc = typename AccT<MODE>::type;
     using V = typename AccT<MODE>::vec;
     using Part = typename AccT<MODE>::part;
+    // BF16 factors with 16 RHS on leaves of up to 192 rows: phase 1 on tensor cores
+    constexpr bool kTensorPhase1 = MODE == 0 && NR == 16 && std::is_same<C, uint16_t>::value && RPL <= 6;
+    constexpr bool MR1 = MODE == 0 && NR > 4 && !kTensorPhase1;  // phase 1 over column groups
     auto* const phase1 = [] {
-        if constexpr (MODE == 0)
+        if constexpr (kTensorPhase1)
+            return k_phase1_tc<NCW>;
+        else if constexpr (MR1)
+            return k_phase1_mr<C, NR, NCW>;
+        else if constexpr (MODE == 0)
             return k_phase1<C, NR, RPL, NCW, ST>;
         else
             return k_phase1_f64<C, NR, RPL, NCW>;
     }();
-    const size_t smem1 = BAR_BYTES + (size_t)ST * STAGE_BYTES + P1_TAIL;
-    // BF16 factors with 16 RHS on leaves of up to 192 rows: phase 1 on tensor cores
-    constexpr bool kTensorPhase1 = MODE == 0 && NR == 16 && std::is_same<C, uint16_t>::value && RPL == 6;
+    const size_t smem1 = BAR_BYTES + (size_t)(MR1 ? MR_STAGES : ST) * STAGE_BYTES + P1_TAIL +
+                         (MR1 ? (size_t)32 * RPL * NR * sizeof(float) : 0);
     // BF16 factors with one RHS: the U slices of phase 2 on tensor cores, which read t in
     // packed BF16 (hi, lo) form (phase 1 stays on the CUDA cores: one mma.sync per 16 x 16
     // tile did not keep up with the stream there)
@@ -1540,8 +1734,8 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
                   "the single-RHS tensor-core phase 2 assumes 16 consumer warps without row split");
     // BF16 factors with 16 RHS: the U slices of phase 2 on tensor cores as well, reading t
     // in the packed BF16 form of k_reduce_pack16_mix
-    constexpr bool kTensorPhase2x16 = MODE == 0 && NR == 16 && std::is_same<C, uint16_t>::value && RPL == 6;
-    constexpr int KP = (MODE == 0 && NR == 16 && RPL == 6) ? 8 : 1;  // RHS per flush pass of k_phase2
+    constexpr bool kTensorPhase2x16 = MODE == 0 && NR == 16 && std::is_same<C, uint16_t>::value && RPL <= 6;
+    constexpr int KP = (MODE == 0 && NR == 16 && RPL <= 6) ? 8 : 1;  // RHS per flush pass of k_phase2
     const size_t smem2 = BAR_BYTES + (size_t)ST * (ZRange<V, NR>::BYTES + STAGE_BYTES) +
                          (size_t)KP * (NCW2 / RS) * 32 * RPL * sizeof(Acc) + (kTensorPhase2x16 ? 16 * 196 * 4 : 0);
     // shared-memory opt-in, once per device for each instantiation
@@ -1550,8 +1744,6 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     HM_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
         HM_CUDA(cudaFuncSetAttribute(phase1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
-        if constexpr (kTensorPhase1)
-            HM_CUDA(cudaFuncSetAttribute(k_phase1_tc<NCW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
         HM_CUDA(cudaFuncSetAttribute(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
@@ -1561,12 +1753,7 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
         a.chunks = PL.ch1.p;
         a.cta_begin = PL.cta1.p;
         a.out = MODE == 0 ? (void*)H.Pf.p : (void*)H.P.p;
-        bool tc = false;
-        if constexpr (kTensorPhase1) tc = base.nr == 16;
-        if (tc)
-            launch_pdl(k_phase1_tc<NCW>, dim3(H.grid), dim3((NCW + 1) * 32), smem1, st, a);
-        else
-            launch_pdl(phase1, dim3(H.grid), dim3((NCW + 1) * 32), smem1, st, a);
+        launch_pdl(phase1, dim3(H.grid), dim3((NCW + 1) * 32), smem1, st, a);
         HM_LAUNCH_CHECK();
         if (timed) mark(H, 2, st);
         using Zt = typename AccT<MODE>::zin;
@@ -1579,23 +1766,19 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
                        (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const int32_t*)H.red_order.p,
                        H.n_red_big, H.n_red,
                        (const Part*)a.out, (uint32_t*)base.tb, base.skip);
-        else if (kTensorPhase2x16 && base.nr == 16)
+        else if constexpr (kTensorPhase2x16)
             launch_pdl(k_reduce_pack16_mix, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
                        (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const int32_t*)H.red_order.p,
                        H.n_red_big, H.n_red, (const float*)a.out, (uint16_t*)base.tb, base.skip);
-        else if (base.nr == 1)
+        else if constexpr (NR == 1)
             launch_pdl(k_reduce_mix<Part, Zt>, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
                        (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const int32_t*)H.red_order.p,
                        H.n_red_big, H.n_red,
                        (const Part*)a.out, (Zt*)base.tb, base.skip);
-        else if (MODE == 0 && (base.nr & 3) == 0)
-            launch_pdl(k_reduce_tb<Part, Zt, MODE == 0>, dim3((unsigned)H.n_far), dim3(128), 0, st,
-                       (const FarDesc*)H.far.p, (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const Part*)a.out,
-                       (Zt*)base.tb, base.nr, base.skip);
         else
-            launch_pdl(k_reduce_tb<Part, Zt, false>, dim3((unsigned)H.n_far), dim3(128), 0, st,
-                       (const FarDesc*)H.far.p, (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const Part*)a.out,
-                       (Zt*)base.tb, base.nr, base.skip);
+            launch_pdl(k_reduce_tb<Part, Zt, MODE == 0>, dim3((unsigned)H.n_far), dim3(128), 0, st,
+                       (const FarDesc*)H.far.p, (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p,
+                       (const Part*)a.out, (Zt*)base.tb, NR, base.skip);
         HM_LAUNCH_CHECK();
         if (timed) mark(H, 3, st);
     } else if (timed) {
@@ -1613,7 +1796,15 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
 
 template <int MODE, class C, int NR>
 void launch_rpl(HMat& H, const HMat::Plan& PL, const StreamArgs& a, bool timed, cudaStream_t st) {
-    if (H.ld_max <= 192)
+    // 16 RHS split a column's rows over two warps, so leaves of at most 128 rows have a
+    // variant of their own: with three row blocks a warp, one of 99 rows left the second warp
+    // one block (three 150 x 150 planes, BF16: phase 2 905 us before, 692 with two and
+    // two and the finer tensor-core mapping;
+    // a split computed from each leaf's rows cost the 176-row leaves of three 100 x 100 planes
+    // 10 %)
+    if (NR == 16 && H.ld_max <= 128) {
+        if constexpr (NR == 16) launch_phases<MODE, C, NR, 4>(H, PL, a, timed, st);
+    } else if (H.ld_max <= 192)
         launch_phases<MODE, C, NR, 6>(H, PL, a, timed, st);
     else
         launch_phases<MODE, C, NR, 12>(H, PL, a, timed, st);
@@ -1649,16 +1840,23 @@ void launch_nr(HMat& H, const HMat::Plan& PL, const StreamArgs& a, int nrhs, boo
             default: fail(HM_EINVAL, "product: 1 to 4 right-hand sides per F64 pass");
         }
     } else {
-        if (nrhs == 1)
-            launch_rpl<MODE, C, 1>(H, PL, a, timed, st);
-        else if (nrhs <= 4)
-            launch_rpl<MODE, C, 4>(H, PL, a, timed, st);
-        else
-            launch_rpl<MODE, C, 16>(H, PL, a, timed, st);
+        switch (nrhs) {
+            case 1: return launch_rpl<MODE, C, 1>(H, PL, a, timed, st);
+            case 4: return launch_rpl<MODE, C, 4>(H, PL, a, timed, st);
+            case 8: return launch_rpl<MODE, C, 8>(H, PL, a, timed, st);
+            case 16: return launch_rpl<MODE, C, 16>(H, PL, a, timed, st);
+            default: fail(HM_EINVAL, "product: 1, 4, 8 or 16 right-hand sides per F32 pass");
+        }
     }
 }
 
-// phase 1, reduction and phase 2 on cluster-ordered operands (see hmat_impl.h)
+// The F32 kernels take 1, 4, 8 or 16 right-hand sides: other counts are padded with zero
+// vectors, whose products are not written.  (The kernels that tested each count in their
+// loops took 3.18 ms for 12 BF16 right-hand sides on three 150 x 150 planes, 1.44 ms for 16.)
+int padded_rhs(int nr) { return nr == 1 ? 1 : (nr <= 4 ? 4 : (nr <= 8 ? 8 : 16)); }
+
+// phase 1, reduction and phase 2 on cluster-ordered operands (see hmat_impl.h); F32: xc
+// interleaved by padded_rhs(nr)
 void run_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, bool timed, cudaStream_t st,
               const int* skip = nullptr) {
     if (!has_factors(H, fac)) fail(HM_EINVAL, "product: the requested factor precision is not stored");
@@ -1671,7 +1869,7 @@ void run_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, boo
     a.counters = H.counters.p;
     a.err = H.err.p;
     a.ndof = H.ndof;
-    a.nr = nr;
+    a.nout = nr;
     a.ld_max = H.ld_max;
     a.skip = skip;
     a.wait_ns = H.wait_ns;
@@ -1685,9 +1883,9 @@ void run_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, boo
                                  : launch_shape_variant<float>(H, PL, a, timed, st)))
             return;
         if (fac == 1)
-            launch_nr<0, uint16_t>(H, PL, a, nr, timed, st);
+            launch_nr<0, uint16_t>(H, PL, a, padded_rhs(nr), timed, st);
         else
-            launch_nr<0, float>(H, PL, a, nr, timed, st);
+            launch_nr<0, float>(H, PL, a, padded_rhs(nr), timed, st);
     } else {
         a.tb = H.tb.p;
         a.slots = H.slotsd.p;
@@ -1855,6 +2053,12 @@ int product_pass(int dtype) { return dtype == HM_F64 ? F64_PASS : 16; }
 void product_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, cudaStream_t st, const int* skip) {
     if (nr < 1 || nr > product_pass(dtype)) fail(HM_EINVAL, "product: too many right-hand sides in one pass");
     ensure_product_scratch(H, nr, st);
+    if (dtype == HM_F32 && padded_rhs(nr) != nr) {
+        const int np = padded_rhs(nr);
+        k_pad<<<(unsigned)ceil_div(H.ndof * np, 256), 256, 0, st>>>((const float*)xc, H.xcf.p, H.ndof, nr, np);
+        HM_LAUNCH_CHECK();
+        xc = H.xcf.p;
+    }
     run_core(H, xc, yc, nr, dtype, fac, false, st, skip);
 }
 
@@ -1878,7 +2082,8 @@ void matvec(HMat& H, const void* x, void* y, int nrhs, int dtype, cudaStream_t s
         if (dtype == HM_F32) {
             const float* xf = (const float*)x + (int64_t)k0 * H.ndof;
             float* yf = (float*)y + (int64_t)k0 * H.ndof;
-            k_gather<float><<<gb, 256, 0, st>>>(xf, H.xcf.p, H.perm.p, H.N, nr);
+            const int np = padded_rhs(nr);
+            k_gather<<<(unsigned)ceil_div(H.ndof * np, 256), 256, 0, st>>>(xf, H.xcf.p, H.perm.p, H.N, nr, np);
             mark(H, 1, st);
             run_core(H, H.xcf.p, H.ycf.p, nr, dtype, fac, true, st);
             launch_pdl(k_scatter<float>, dim3(gb), dim3(256), 0, st, (const float*)H.ycf.p, yf,

@@ -43,3 +43,30 @@ def test_f64_passes_match_single_rhs(leaf, storage):
         err = np.linalg.norm((y - one[:nrhs]).cpu().numpy(), axis=1) / scale[:nrhs]
         assert err.max() <= 1e-11, (nrhs, err)
     H.check()
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("leaf", [8, 33, 42, 64, 110])
+def test_f32_counts_match_f64_vectors(leaf, storage):
+    """FP32 vectors, every count a pass is padded from (2 .. 16) and counts cut into several
+    passes, against the FP64-vector product of the same stored factors: every right-hand side
+    within 1e-5 of its absolute sums (FP32 accumulation, and 16 bits of the vectors on the
+    tensor-core paths: the bar of the served paths' tests)."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    el = synth.disk_mesh(26)
+    T = hmat.ClusterTree(el, leaf, 1.0)
+    H = hmat.HMatrix(T, el, E, NU, 1e-6, storage)
+    A = np.abs(O.dense_matrix(el, E, NU))
+    X = synth.rhs_normal(3 * el.N, 71 + leaf, 19).astype(np.float32)
+    x = torch.from_numpy(X).cuda()
+    ref = torch.empty((19, 3 * el.N), dtype=torch.float64, device="cuda")
+    H.matvec(x.double(), ref)
+    scale = np.linalg.norm(A @ np.abs(X).T.astype(np.float64), axis=0)
+    for nrhs in (1, 2, 3, 4, 5, 8, 9, 15, 16, 17, 19):
+        y = torch.full((nrhs, 3 * el.N), float("nan"), dtype=torch.float32, device="cuda")
+        H.matvec(x[:nrhs].contiguous(), y)
+        err = np.linalg.norm((y.double() - ref[:nrhs]).cpu().numpy(), axis=1) / scale[:nrhs]
+        assert err.max() <= 1e-5, (nrhs, err)
+    H.check()
