@@ -1035,7 +1035,7 @@ def main():
                        "assemble_coeff_blocks": info["coeff_blocks"],
                        "rank_mean": info["rank_mean"], "rank_max": info["rank_max"],
                        "bytes_per_product": B, "frac_of_hbm_peak": value / world / hbm},
-            "roofline": roofline, "e2e": e2e, "gpu_launches": 5 * args.steps, "clocks": clocks,
+            "roofline": roofline, "e2e": e2e, "gpu_launches": 4 * args.steps, "clocks": clocks,
             "f64_vectors_compensated": f64_vectors}
     if gmres is not None:
         line["gmres"] = gmres

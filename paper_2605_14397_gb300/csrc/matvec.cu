@@ -4,8 +4,8 @@
 //   gather   xc = x[perm]                          cluster order, RHS interleaved
 //   phase 1  P = V_t^T xc_t                        every V column (one per rank per leaf)
 //   reduce   tb_b = sum of the partials of block b over the leaves of its column cluster
-//   phase 2  yc_s = [D_s | U_s] z_s, z = xc (near columns) or tb (U columns)
-//   scatter  y[perm] = yc
+//   phase 2  y_s = [D_s | U_s] z_s, z = xc (near columns) or tb (U columns), written to
+//            y[perm] (the solvers keep cluster order)
 //
 // Phases 1 and 2 are persistent kernels, one CTA per SM.  Their coefficient streams are
 // cut into chunks of whole columns of one tile or factor slice (at most 32 KB and 128
@@ -275,19 +275,6 @@ __global__ void k_gather_split(const double* __restrict__ x, float2* __restrict_
     const int64_t r = q / nrhs, k = q % nrhs;
     const int64_t p = r / 3, m = r % 3;
     xc[q] = split_d(x[k * ndof + 3 * (int64_t)perm[p] + m]);
-}
-
-// y[k * ndof + user dof] = yc[k * ndof + dof]
-template <class V>
-__global__ void k_scatter(const V* __restrict__ yc, V* __restrict__ y, const int32_t* __restrict__ perm, int64_t N,
-                          int nrhs) {
-    pdl_wait();
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t ndof = 3 * N;
-    if (q >= ndof * nrhs) return;
-    const int64_t k = q / ndof, r = q % ndof;
-    const int64_t p = r / 3, m = r % 3;
-    y[k * ndof + 3 * (int64_t)perm[p] + m] = yc[q];
 }
 
 __device__ __forceinline__ float to_zin(float v, float*) { return v; }
@@ -645,6 +632,7 @@ struct StreamArgs {
     void* slots;  // phase-2 partials of split leaves
     int32_t* counters;
     int* err;
+    const int32_t* perm;  // phase 2: rows of out in user order (cluster position -> element); NULL: cluster order
     int64_t ndof;
     int nout;     // right-hand sides the caller asked for (the vectors of out); the rest pad the kernel's count
     int ld_max;
@@ -908,6 +896,12 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     int cur = -1, rot = 0;
     LeafDesc L{};
 
+    // entry r of the leaf in an output vector (matvec's y in user order: the permutation costs
+    // the flush a cached load, a kernel of its own over y cost 3 to 6 us a product)
+    auto out_at = [&](int k, int r) -> Vv& {
+        const int64_t p = (int64_t)L.begin + r / 3;
+        return yc[(int64_t)k * a.ndof + 3 * (a.perm ? (int64_t)a.perm[p] : p) + r % 3];
+    };
     auto flush = [&]() {
         const LeafSplit sp = a.split[cur];
         const int rows = 3 * L.n;
@@ -949,7 +943,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
                 for (int q = 1; q < NG; ++q) acc_add(s, rk[(size_t)q * (32 * RPL) + r]);
                 if constexpr (TC16) acc_add(s, ty[(size_t)k * TY_LD + r]);
                 if (whole)
-                    yc[(int64_t)k * a.ndof + 3 * (int64_t)L.begin + r] = (Vv)acc_value(s);
+                    out_at(k, r) = (Vv)acc_value(s);
                 else
                     slots[(slot * NR + k) * a.ld_max + r] = (Vv)acc_value(s);
             }
@@ -970,7 +964,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
                         Vv s = 0;
                         for (int p = 0; p < sp.nparts; ++p)
                             s += __ldcg(slots + ((int64_t)(sp.slot_base + p) * NR + k) * a.ld_max + r);
-                        yc[(int64_t)k * a.ndof + 3 * (int64_t)L.begin + r] = s;
+                        out_at(k, r) = s;
                     }
                 if (threadIdx.x == 0) a.counters[cur] = 0;
             }
@@ -1856,9 +1850,9 @@ void launch_nr(HMat& H, const HMat::Plan& PL, const StreamArgs& a, int nrhs, boo
 int padded_rhs(int nr) { return nr == 1 ? 1 : (nr <= 4 ? 4 : (nr <= 8 ? 8 : 16)); }
 
 // phase 1, reduction and phase 2 on cluster-ordered operands (see hmat_impl.h); F32: xc
-// interleaved by padded_rhs(nr)
+// interleaved by padded_rhs(nr).  perm: yc in user order.
 void run_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, bool timed, cudaStream_t st,
-              const int* skip = nullptr) {
+              const int* skip = nullptr, const int32_t* perm = nullptr) {
     if (!has_factors(H, fac)) fail(HM_EINVAL, "product: the requested factor precision is not stored");
     const HMat::Plan& PL = H.plan[fac];
     StreamArgs a{};
@@ -1870,6 +1864,7 @@ void run_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, boo
     a.err = H.err.p;
     a.ndof = H.ndof;
     a.nout = nr;
+    a.perm = perm;
     a.ld_max = H.ld_max;
     a.skip = skip;
     a.wait_ns = H.wait_ns;
@@ -2085,17 +2080,13 @@ void matvec(HMat& H, const void* x, void* y, int nrhs, int dtype, cudaStream_t s
             const int np = padded_rhs(nr);
             k_gather<<<(unsigned)ceil_div(H.ndof * np, 256), 256, 0, st>>>(xf, H.xcf.p, H.perm.p, H.N, nr, np);
             mark(H, 1, st);
-            run_core(H, H.xcf.p, H.ycf.p, nr, dtype, fac, true, st);
-            launch_pdl(k_scatter<float>, dim3(gb), dim3(256), 0, st, (const float*)H.ycf.p, yf,
-                       (const int32_t*)H.perm.p, (int64_t)H.N, nr);
+            run_core(H, H.xcf.p, yf, nr, dtype, fac, true, st, nullptr, H.perm.p);
         } else {
             const double* xd = (const double*)x + (int64_t)k0 * H.ndof;
             double* yd = (double*)y + (int64_t)k0 * H.ndof;
             k_gather_split<<<gb, 256, 0, st>>>(xd, (float2*)H.xc.p, H.perm.p, H.N, nr);
             mark(H, 1, st);
-            run_core(H, H.xc.p, H.yc.p, nr, dtype, fac, true, st);
-            launch_pdl(k_scatter<double>, dim3(gb), dim3(256), 0, st, (const double*)H.yc.p, yd,
-                       (const int32_t*)H.perm.p, (int64_t)H.N, nr);
+            run_core(H, H.xc.p, yd, nr, dtype, fac, true, st, nullptr, H.perm.p);
         }
         HM_LAUNCH_CHECK();
         mark(H, 5, st);
