@@ -30,6 +30,7 @@
 #include "hmat_impl.h"
 #include "ilu_dev.h"
 #include "learned.h"
+#include "warp_sums.cuh"
 
 namespace hm {
 
@@ -37,6 +38,10 @@ namespace {
 
 constexpr int ROW_NT = 256;
 constexpr int ROWS_PER_CTA = 1024;  // 4 rows per thread
+// Rows per thread of the Arnoldi kernels: four, or one where that would leave SMs without a
+// CTA (fewer than 152 x 1,024 rows): their length is then a chain of loads and warp sums over
+// the basis, which more CTAs do not lengthen.
+int arnoldi_rows(int64_t ndof) { return ndof < (int64_t)152 * ROWS_PER_CTA ? 1 : 4; }
 constexpr int VSLACK = 64;          // elements after each buffer read by rounded copies
 constexpr int BJ_MAX_ROWS_SMEM = 224;
 
@@ -634,16 +639,31 @@ __global__ void __launch_bounds__(256) k_bj_apply(const LeafDesc* __restrict__ l
         float acc[12];
 #pragma unroll
         for (int i = 0; i < 12; ++i) acc[i] = 0.f;
-        // two columns per pass: twice the loads in flight
+        // four columns per pass: their loads are in flight together
         int c = w;
-        for (; c + 8 < n; c += 16) {
-            const float vc0 = (float)vk[c], vc1 = (float)vk[c + 8];
-            const float* col0 = B + (int64_t)c * L.ld;
-            const float* col1 = col0 + (int64_t)8 * L.ld;
+        for (; c + 24 < n; c += 32) {
+            float vc[4];
+            const float* col[4];
 #pragma unroll
-            for (int i = 0; i < 12; ++i) {
-                const int r = lane + 32 * i;
-                if (r < n) acc[i] = fmaf(__ldg(col1 + r), vc1, fmaf(__ldg(col0 + r), vc0, acc[i]));
+            for (int q = 0; q < 4; ++q) {
+                vc[q] = (float)vk[c + 8 * q];
+                col[q] = B + (int64_t)(c + 8 * q) * L.ld;
+            }
+#pragma unroll
+            for (int i0 = 0; i0 < 12; i0 += 6) {
+                if (32 * i0 >= n) break;
+                float b[6][4];
+#pragma unroll
+                for (int i = 0; i < 6; ++i)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int r = lane + 32 * (i0 + i);
+                        b[i][q] = r < n ? __ldg(col[q] + r) : 0.f;
+                    }
+#pragma unroll
+                for (int i = 0; i < 6; ++i)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) acc[i0 + i] = fmaf(b[i][q], vc[q], acc[i0 + i]);
             }
         }
         for (; c < n; c += 8) {
@@ -930,8 +950,31 @@ __global__ void k_to_f32_interleaved(const double* __restrict__ in, float* __res
 template <class Y>
 __device__ __forceinline__ double yval(const Y* y, int64_t i) { return (double)y[i]; }
 
+// partial dots over a CTA's rows of w (wl: U rows a thread from r0) with V_0 .. V_j of RHS k,
+// per warp into sp; four basis vectors a pass, whose warp sums share one butterfly
+template <int U>
+__device__ __forceinline__ void basis_dots(const double* __restrict__ V, int64_t vstride, int nr, int k, int j,
+                                           const double (&wl)[U], int64_t r0, int64_t ndof, double (*sp)[132]) {
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    for (int j0 = 0; j0 <= j; j0 += 4) {
+        double d[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const double* Vj = V + ((int64_t)min(j0 + q, j) * nr + k) * vstride;
+            d[q] = 0.0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t i = r0 + threadIdx.x + u * ROW_NT;
+                if (i < ndof) d[q] += Vj[i] * wl[u];
+            }
+        }
+        const int q = warp_sums<4>(d, lane);
+        if ((lane & 7) == 0 && j0 + q <= j) sp[wp][j0 + q] = d[0];
+    }
+}
+
 // pass 1: w = y - d .* z (stored), partial dots with V_0..V_j
-template <class Y>
+template <class Y, int U>
 __global__ void __launch_bounds__(ROW_NT) k_arn_first(const Y* __restrict__ y, const double* __restrict__ d,
                                                       const double* __restrict__ blk,
                                                       const double* __restrict__ z, double* __restrict__ w,
@@ -939,13 +982,12 @@ __global__ void __launch_bounds__(ROW_NT) k_arn_first(const Y* __restrict__ y, c
                                                       int64_t vstride, double* __restrict__ part,
                                                       const CycleState* __restrict__ cs) {
     __shared__ double sp[ROW_NT / 32][132];
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const int64_t r0 = (int64_t)blockIdx.x * ROWS_PER_CTA;
+    const int64_t r0 = (int64_t)blockIdx.x * (ROW_NT * U);
     for (int k = 0; k < nr; ++k) {
         if (cs[k].done) continue;
-        double wl[4];
+        double wl[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
             const int64_t i = r0 + threadIdx.x + u * ROW_NT;
             double v = 0.0;
             if (i < ndof) {
@@ -955,17 +997,7 @@ __global__ void __launch_bounds__(ROW_NT) k_arn_first(const Y* __restrict__ y, c
             }
             wl[u] = v;
         }
-        for (int jj = 0; jj <= j; ++jj) {
-            const double* Vj = V + ((int64_t)jj * nr + k) * vstride;
-            double s = 0.0;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t i = r0 + threadIdx.x + u * ROW_NT;
-                if (i < ndof) s += Vj[i] * wl[u];
-            }
-            s = warp_sum_d(s);
-            if (lane == 0) sp[wp][jj] = s;
-        }
+        basis_dots<U>(V, vstride, nr, k, j, wl, r0, ndof, sp);
         __syncthreads();
         for (int jj = threadIdx.x; jj <= j; jj += ROW_NT) {
             double s = 0.0;
@@ -1005,6 +1037,7 @@ __global__ void k_reduce_parts(const double* __restrict__ part, int nblk, int nr
 
 // w -= V h (h = previous dots); then either partial dots with V (second pass) or
 // the partial squared norm of w (last pass)
+template <int U>
 __global__ void __launch_bounds__(ROW_NT) k_arn_update(double* __restrict__ w, const double* __restrict__ V,
                                                        const double* __restrict__ h, int64_t ndof, int nr, int j,
                                                        int64_t vstride, double* __restrict__ part, int want_dots,
@@ -1012,37 +1045,30 @@ __global__ void __launch_bounds__(ROW_NT) k_arn_update(double* __restrict__ w, c
     __shared__ double sp[ROW_NT / 32][132];
     __shared__ double sh[132];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const int64_t r0 = (int64_t)blockIdx.x * ROWS_PER_CTA;
+    const int64_t r0 = (int64_t)blockIdx.x * (ROW_NT * U);
     for (int k = 0; k < nr; ++k) {
         if (cs[k].done) continue;
         for (int jj = threadIdx.x; jj <= j; jj += ROW_NT) sh[jj] = h[k * 132 + jj];
         __syncthreads();
-        double wl[4];
+        double wl[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
             const int64_t i = r0 + threadIdx.x + u * ROW_NT;
             double v = 0.0;
             if (i < ndof) {
                 v = w[k * ndof + i];
+#pragma unroll 4
                 for (int jj = 0; jj <= j; ++jj) v -= V[((int64_t)jj * nr + k) * vstride + i] * sh[jj];
                 w[k * ndof + i] = v;
             }
             wl[u] = v;
         }
         if (want_dots) {
-            for (int jj = 0; jj <= j; ++jj) {
-                const double* Vj = V + ((int64_t)jj * nr + k) * vstride;
-                double s = 0.0;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int64_t i = r0 + threadIdx.x + u * ROW_NT;
-                    if (i < ndof) s += Vj[i] * wl[u];
-                }
-                s = warp_sum_d(s);
-                if (lane == 0) sp[wp][jj] = s;
-            }
+            basis_dots<U>(V, vstride, nr, k, j, wl, r0, ndof, sp);
         } else {
-            double s = wl[0] * wl[0] + wl[1] * wl[1] + wl[2] * wl[2] + wl[3] * wl[3];
+            double s = 0.0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) s += wl[u] * wl[u];
             s = warp_sum_d(s);
             if (lane == 0) sp[wp][0] = s;
         }
@@ -1449,8 +1475,7 @@ SolveWS& workspace(HMat& H, int nr, int m, cudaStream_t st) {
     W.sn.alloc((size_t)W.nr * (W.m + 1));
     W.g.alloc((size_t)W.nr * (W.m + 1));
     W.ylsq.alloc((size_t)W.nr * (W.m + 1));
-    const int nb = nblk_rows(H.ndof);
-    W.part.alloc((size_t)nb * W.nr * 132);
+    W.part.alloc((size_t)ceil_div(H.ndof, ROW_NT * arnoldi_rows(H.ndof)) * W.nr * 132);
     W.h1.alloc((size_t)W.nr * 132);
     W.h2.alloc((size_t)W.nr * 132);
     W.st.alloc(W.nr);
@@ -1542,7 +1567,12 @@ CycleResult fgmres_cycle(HMat& H, SolveWS& W, const double* beta_h, const double
                          int nr, int m, int dtype, int fac, PcKind pc, cudaStream_t st) {
     NvtxScope nvtx_("fgmres_cycle");
     const int64_t n = H.ndof;
-    const int nb = nblk_rows(n);
+    const bool one = arnoldi_rows(n) == 1;
+    const int nb = (int)ceil_div(n, ROW_NT * arnoldi_rows(n));
+    auto update = [&](const double* h, int j, int want_dots) {
+        (one ? k_arn_update<1> : k_arn_update<4>)<<<nb, ROW_NT, 0, st>>>(W.w.p, W.V.p, h, n, nr, j, W.vstride, W.part.p,
+                                                                         want_dots, W.st.p);
+    };
     std::vector<CycleState> cs(nr);
     for (int k = 0; k < nr; ++k) {
         cs[k].done = active_h[k] ? 0 : 1;
@@ -1571,18 +1601,20 @@ CycleResult fgmres_cycle(HMat& H, SolveWS& W, const double* beta_h, const double
         precond_apply(H, W, pc, vj, zj, dtype == HM_F32 ? W.zf.p : nullptr, nr, st);
         if (dtype == HM_F64) {
             apply_E(H, W, zj, nullptr, W.y64.p, nr, HM_F64, fac, st, W.alldone.p);
-            k_arn_first<double><<<nb, ROW_NT, 0, st>>>(W.y64.p, W.dc.p, W.blk, zj, W.w.p, W.V.p, n, nr, j, W.vstride,
+            (one ? k_arn_first<double, 1> : k_arn_first<double, 4>)<<<nb, ROW_NT, 0, st>>>(
+                W.y64.p, W.dc.p, W.blk, zj, W.w.p, W.V.p, n, nr, j, W.vstride,
                                                        W.part.p, W.st.p);
         } else {
             apply_E(H, W, nullptr, W.zf.p, W.y32.p, nr, HM_F32, fac, st, W.alldone.p);
-            k_arn_first<float><<<nb, ROW_NT, 0, st>>>(W.y32.p, W.dc.p, W.blk, zj, W.w.p, W.V.p, n, nr, j, W.vstride,
+            (one ? k_arn_first<float, 1> : k_arn_first<float, 4>)<<<nb, ROW_NT, 0, st>>>(
+                W.y32.p, W.dc.p, W.blk, zj, W.w.p, W.V.p, n, nr, j, W.vstride,
                                                       W.part.p, W.st.p);
         }
         HM_LAUNCH_CHECK();
         k_reduce_parts<<<nr, 512, 0, st>>>(W.part.p, nb, nr, j + 1, W.h1.p, W.st.p);
-        k_arn_update<<<nb, ROW_NT, 0, st>>>(W.w.p, W.V.p, W.h1.p, n, nr, j, W.vstride, W.part.p, 1, W.st.p);
+        update(W.h1.p, j, 1);
         k_reduce_parts<<<nr, 512, 0, st>>>(W.part.p, nb, nr, j + 1, W.h2.p, W.st.p);
-        k_arn_update<<<nb, ROW_NT, 0, st>>>(W.w.p, W.V.p, W.h2.p, n, nr, j, W.vstride, W.part.p, 0, W.st.p);
+        update(W.h2.p, j, 0);
         k_givens<<<1, 32, 0, st>>>(W.h1.p, W.h2.p, W.part.p, nb, nr, j, m, W.Hm.p, W.cs.p, W.sn.p, W.g.p, W.st.p,
                                    W.alldone.p);
         k_scale_next<<<g1(n * nr), 256, 0, st>>>(W.w.p, W.V.p, n, nr, j, W.vstride, W.st.p);
