@@ -206,7 +206,7 @@ def time_gmres(H, el, dev, torch, reps=3):
 
 def run_faults64(args, dev, torch, hmat, synth):
     """64 independent disk faults (log-uniform 2k-40k elements, seeded normals and nu,
-    795,192 elements in all): one batched H-matrix (one work list, 5 launches per
+    795,192 elements in all): one batched H-matrix (one work list, 4 launches per
     product; also replayed from a CUDA graph) against per-fault products (64 x 5
     launches; also 64 graph replays).  value = algorithmic bytes of all 64 products /
     time of the batched product."""

@@ -230,8 +230,8 @@ hm_status hm_matvec_host(const hm_hmat* h, const void* x_host, void* y_host, int
  * stream between the phases.  enable = 1 clears the accumulators and starts recording,
  * enable = 0 stops.  hm_hmat_timing_read synchronises with the last recorded event and
  * returns, in milliseconds summed over the timed products: out[0] gather, out[1] phase 1
- * (V^T x), out[2] reduction of the partials, out[3] phase 2 ([D | U] z), out[4] 0 (phase 2 writes user order),
- * and out[5] the number of timed products. */
+ * (V^T x), out[2] reduction of the partials, out[3] phase 2 ([D | U] z), out[4] the end of the
+ * product (no kernel: phase 2 writes user order), and out[5] the number of timed products. */
 hm_status hm_hmat_timing(const hm_hmat* h, int enable);
 hm_status hm_hmat_timing_read(const hm_hmat* h, double* out6);
 

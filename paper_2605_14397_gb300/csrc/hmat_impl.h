@@ -193,8 +193,8 @@ struct HMat {
 
     // product scratch, sized for nrhs_cap right-hand sides
     int nrhs_cap = 0;
-    DevBuf<double> xc, yc;        // cluster-order vectors (F64 path) [nrhs][ndof]
-    DevBuf<float> xcf, ycf;       // (F32 path)
+    DevBuf<double> xc;            // cluster-order operands (F64 path, (hi, lo) floats) [ndof][nrhs]
+    DevBuf<float> xcf;            // (F32 path)
     DevBuf<double> P, tb;         // partials / t vectors (F64 path uses hi+lo pairs as double)
     DevBuf<float> Pf, tbf;
 

@@ -66,22 +66,19 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 
 template <int MODE>
 struct AccT;
-// type: accumulator; vec: output vectors (y); part: phase-1 partials as they are stored;
-// zin: the x / t operands as the kernels read them -- in F64 mode each double is stored
-// pre-split into (hi, lo) floats by the gather and the reduction, and the partials are the
-// accumulators themselves, so the streaming kernels do no FP64 arithmetic
+// type: accumulator; vec: output vectors (y, partials); zin: the x / t operands as the
+// kernels read them -- in F64 mode each double is stored pre-split into (hi, lo) floats
+// by the gather and the reduction, so the streaming kernels do no FP64 arithmetic
 template <>
 struct AccT<0> {
     using type = float;
     using vec = float;
-    using part = float;
     using zin = float;
 };
 template <>
 struct AccT<1> {
     using type = FF;
     using vec = double;
-    using part = float2;
     using zin = float2;
 };
 
@@ -182,11 +179,6 @@ __device__ __forceinline__ int warp_reduce_scatter(Acc (&acc)[NR], int lane) {
 
 __device__ __forceinline__ float acc_value(float a) { return a; }
 __device__ __forceinline__ double acc_value(const FF& a) { return (double)a.hi + (double)a.lo; }
-// a phase-1 partial as the reduction adds it
-__device__ __forceinline__ float part_value(float a) { return a; }
-__device__ __forceinline__ double part_value(float2 a) { return (double)a.x + (double)a.y; }
-template <class Part>
-using PartSum = decltype(part_value(Part()));
 
 // the (hi, lo) operands of one column for NR right-hand sides in F64 mode (16-byte aligned
 // for an even NR)
@@ -291,11 +283,10 @@ __device__ __forceinline__ uint32_t to_zin(float v, uint32_t*) {
 // per block: the n = r nr entries times G = 128 / n interleaved groups of leaf partials,
 // four independent loads in flight per thread, groups combined in a fixed order.  In F64
 // mode the sums are stored as (hi, lo) float pairs, the form phase 2 reads.
-template <class Part, class Zt, bool VEC4>
+template <class V, class Zt, bool VEC4>
 __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ far, const int32_t* __restrict__ poff,
-                                                   const int32_t* __restrict__ uoff, const Part* __restrict__ P,
+                                                   const int32_t* __restrict__ uoff, const V* __restrict__ P,
                                                    Zt* __restrict__ tb, int nrhs, const int* __restrict__ skip) {
-    using V = PartSum<Part>;
     __shared__ V sp[128];
     pdl_wait();
     pdl_trigger();
@@ -352,12 +343,12 @@ __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ f
             V s0 = 0, s1 = 0, s2 = 0, s3 = 0;
             int q = 0;
             for (; q + 3 < F.n_tleaves; q += 4) {
-                s0 += part_value(P[at(q) + e]);
-                s1 += part_value(P[at(q + 1) + e]);
-                s2 += part_value(P[at(q + 2) + e]);
-                s3 += part_value(P[at(q + 3) + e]);
+                s0 += P[at(q) + e];
+                s1 += P[at(q + 1) + e];
+                s2 += P[at(q + 2) + e];
+                s3 += P[at(q + 3) + e];
             }
-            for (; q < F.n_tleaves; ++q) s0 += part_value(P[at(q) + e]);
+            for (; q < F.n_tleaves; ++q) s0 += P[at(q) + e];
             const Zt t = to_zin((s0 + s1) + (s2 + s3), tb);
             for (int c = 0; c < F.n_sleaves; ++c) tb[(int64_t)uoff[F.ubase + c] * nrhs + e] = t;
         }
@@ -369,12 +360,12 @@ __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ f
     if (g < G) {
         int q = g;
         for (; q + 3 * G < F.n_tleaves; q += 4 * G) {
-            s0 += part_value(P[at(q) + e]);
-            s1 += part_value(P[at(q + G) + e]);
-            s2 += part_value(P[at(q + 2 * G) + e]);
-            s3 += part_value(P[at(q + 3 * G) + e]);
+            s0 += P[at(q) + e];
+            s1 += P[at(q + G) + e];
+            s2 += P[at(q + 2 * G) + e];
+            s3 += P[at(q + 3 * G) + e];
         }
-        for (; q < F.n_tleaves; q += G) s0 += part_value(P[at(q) + e]);
+        for (; q < F.n_tleaves; q += G) s0 += P[at(q) + e];
     }
     sp[threadIdx.x] = (s0 + s1) + (s2 + s3);
     __syncthreads();
@@ -403,14 +394,13 @@ __device__ __forceinline__ int tb16_piece_pos(int64_t l, int q) { return q ^ (in
 // the rank entries, one load fetches 32 offset-table entries which shuffles broadcast.
 // Every block sums its partials in a fixed order.
 constexpr int RED_WARP_LEAVES = 32;
-template <class Part, class Zt>
+template <class V, class Zt>
 __global__ void __launch_bounds__(256) k_reduce_mix(const FarDesc* __restrict__ far,
                                                     const int32_t* __restrict__ poff,
                                                     const int32_t* __restrict__ uoff,
                                                     const int32_t* __restrict__ order, int64_t n_big, int64_t n_all,
-                                                    const Part* __restrict__ P, Zt* __restrict__ tb,
+                                                    const V* __restrict__ P, Zt* __restrict__ tb,
                                                     const int* __restrict__ skip) {
-    using V = PartSum<Part>;
     __shared__ V sp[256];
     constexpr int SPO = 2048;
     __shared__ int32_t spo[SPO];
@@ -432,12 +422,12 @@ __global__ void __launch_bounds__(256) k_reduce_mix(const FarDesc* __restrict__ 
         if (g < G) {
             int q = g;
             for (; q + 3 * G < nt; q += 4 * G) {
-                s0 += part_value(P[(int64_t)po[q] + e]);
-                s1 += part_value(P[(int64_t)po[q + G] + e]);
-                s2 += part_value(P[(int64_t)po[q + 2 * G] + e]);
-                s3 += part_value(P[(int64_t)po[q + 3 * G] + e]);
+                s0 += P[(int64_t)po[q] + e];
+                s1 += P[(int64_t)po[q + G] + e];
+                s2 += P[(int64_t)po[q + 2 * G] + e];
+                s3 += P[(int64_t)po[q + 3 * G] + e];
             }
-            for (; q < nt; q += G) s0 += part_value(P[(int64_t)po[q] + e]);
+            for (; q < nt; q += G) s0 += P[(int64_t)po[q] + e];
         }
         sp[threadIdx.x] = (s0 + s1) + (s2 + s3);
         __syncthreads();
@@ -469,15 +459,15 @@ __global__ void __launch_bounds__(256) k_reduce_mix(const FarDesc* __restrict__ 
                 const int32_t o0 = __shfl_sync(0xffffffffu, mine, q), o1 = __shfl_sync(0xffffffffu, mine, q + 1);
                 const int32_t o2 = __shfl_sync(0xffffffffu, mine, q + 2), o3 = __shfl_sync(0xffffffffu, mine, q + 3);
                 if (on) {
-                    s0 += part_value(P[(int64_t)o0 + e]);
-                    s1 += part_value(P[(int64_t)o1 + e]);
-                    s2 += part_value(P[(int64_t)o2 + e]);
-                    s3 += part_value(P[(int64_t)o3 + e]);
+                    s0 += P[(int64_t)o0 + e];
+                    s1 += P[(int64_t)o1 + e];
+                    s2 += P[(int64_t)o2 + e];
+                    s3 += P[(int64_t)o3 + e];
                 }
             }
             for (; q < m; ++q) {
                 const int32_t o0 = __shfl_sync(0xffffffffu, mine, q);
-                if (on) s0 += part_value(P[(int64_t)o0 + e]);
+                if (on) s0 += P[(int64_t)o0 + e];
             }
         }
         if (on) {
@@ -1415,18 +1405,32 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_mr(StreamArgs a) {
 // four columns for one RHS, two for two, one for three or four -- packed in pairs (over
 // the columns for one RHS, over the RHS otherwise) for the packed FP32 instructions; the
 // four sums over the warp share one reduce-scatter.  The leaf's operands stay in registers
-// already split.  Partials are stored as the (hi, lo) accumulators: adding the two in FP64
-// here, with a few lanes active, had kept the FP64 pipe a third busy; the reduction, which
-// waits on memory, does it with full warps.  Rows past a leaf meet x = 0, and NA, the row
-// blocks of 32 the leaf really has, is a template argument of the column loop.
+// already split.  A partial leaves as a double, hi + lo added in FP64; eight passes wait for
+// that (HeldParts), a lane of every eight holding each, so that the addition fills its warp:
+// one pass at a time it had kept the FP64 pipe a third busy.  Rows past a leaf meet x = 0,
+// and NA, the row blocks of 32 the leaf really has, is a template argument of the column
+// loop.
 // Bound by the FP32 pipe and its issue (a packed instruction takes the pipe two cycles, so
 // packing saves issue slots, not pipe time).  One RHS, 25,700 triangles (444 MB of V,
 // 65 us at the copy bandwidth): 116 us with scalar operations over 192 rows, 104 us packed
-// over the leaf's row blocks, 92 us with the columns dealt across chunks (deal_start).
+// over the leaf's row blocks, 92 us with the columns dealt across chunks (deal_start); the
+// whole product 358 us before, 309 now.
+struct HeldParts {
+    FF v;
+    int64_t at;  // entry of P; -1: none
+    int n;       // passes held
+    __device__ __forceinline__ void store(double* P) {
+        if (at >= 0) P[at] = acc_value(v);
+        at = -1;
+        n = 0;
+    }
+};
+
 constexpr int ff_phase1_group(int NR) { return NR == 1 ? 4 : (NR == 2 ? 2 : 1); }  // columns per pass
 template <int NA, int NR, int RPL, class C, class Ld>
 __device__ __forceinline__ void ff_phase1_columns(const float2 (&x)[NR][RPL], const C* buf, int ld, int u0, int ncw,
-                                                  int ncols, int lane, float2* out, Ld load) {
+                                                  int ncols, int lane, int64_t zoff, double* P, HeldParts& held,
+                                                  Ld load) {
     constexpr int CG = ff_phase1_group(NR);
     for (int c = CG * u0; c < ncols; c += CG * ncw) {
         FF2 acc[2];
@@ -1465,7 +1469,11 @@ __device__ __forceinline__ void ff_phase1_columns(const float2 (&x)[NR][RPL], co
         }
         const int m = warp_reduce_scatter<4>(q, lane);  // value m: column m (one RHS), m / NR (two), RHS m (more)
         const int cj = c + (NR == 1 ? m : (NR == 2 ? m >> 1 : 0)), k = NR == 1 ? 0 : (NR == 2 ? m & 1 : m);
-        if ((lane & 7) == 0 && cj < ncols && k < NR) out[(int64_t)cj * NR + k] = make_float2(q[0].hi, q[0].lo);
+        if ((lane & 7) == held.n) {  // all eight lanes of a group have the sum
+            held.v = q[0];
+            held.at = cj < ncols && k < NR ? (zoff + cj) * NR + k : -1;
+        }
+        if (++held.n == 8) held.store(P);
     }
 }
 
@@ -1492,7 +1500,8 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_f64(StreamArgs a) 
         return;
     }
     pdl_wait();  // x in cluster order comes from the preceding kernel
-    float2* P = (float2*)a.out;
+    double* P = (double*)a.out;
+    HeldParts held{FF{0.f, 0.f}, -1, 0};
     const float2* xs = (const float2*)a.xc;
     int cur = -1, rows = 0, rot = 0;
     float2 x[NR][RPL];
@@ -1516,22 +1525,22 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_f64(StreamArgs a) 
         }
         mbar_wait(full + s, (uint32_t)(q / STAGES) & 1u, a.err, 1, a.wait_ns);
         const C* buf = (const C*)(stage + (size_t)s * STAGE_BYTES);
-        float2* out = P + ch.zoff * NR;
         const int u0 = deal_start<NCW>(w, rot);
         rot = deal_next<NCW>(rot, (ch.ncols + ff_phase1_group(NR) - 1) / ff_phase1_group(NR));
         if constexpr (RPL == 6) {
             if (rows <= 128)
-                ff_phase1_columns<4, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, out, load);
+                ff_phase1_columns<4, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, ch.zoff, P, held, load);
             else if (rows <= 160)
-                ff_phase1_columns<5, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, out, load);
+                ff_phase1_columns<5, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, ch.zoff, P, held, load);
             else
-                ff_phase1_columns<6, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, out, load);
+                ff_phase1_columns<6, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, ch.zoff, P, held, load);
         } else {
-            ff_phase1_columns<RPL, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, out, load);
+            ff_phase1_columns<RPL, NR, RPL>(x, buf, ch.ld, u0, NCW, ch.ncols, lane, ch.zoff, P, held, load);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(empty + s);
     }
+    held.store(P);
 }
 
 // ---- phase 1 on tensor cores: BF16 V factors, 16 right-hand sides
@@ -1704,7 +1713,6 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     static_assert(MODE == 0 || (NR <= F64_PASS && ST == STAGES), "F64 passes");
     using Acc = typename AccT<MODE>::type;
     using V = typename AccT<MODE>::vec;
-    using Part = typename AccT<MODE>::part;
     // BF16 factors with 16 RHS on leaves of up to 192 rows: phase 1 on tensor cores
     constexpr bool kTensorPhase1 = MODE == 0 && NR == 16 && std::is_same<C, uint16_t>::value && RPL <= 6;
     constexpr bool MR1 = MODE == 0 && NR > 4 && !kTensorPhase1;  // phase 1 over column groups
@@ -1756,23 +1764,23 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
         // one RHS: big blocks a CTA each, the others a warp each (red_order)
         const unsigned gm = (unsigned)std::max<int64_t>(1, H.n_red_big + (H.n_red - H.n_red_big + 7) / 8);
         if constexpr (kTensorPhase2x1)
-            launch_pdl(k_reduce_mix<Part, uint32_t>, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
+            launch_pdl(k_reduce_mix<V, uint32_t>, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
                        (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const int32_t*)H.red_order.p,
                        H.n_red_big, H.n_red,
-                       (const Part*)a.out, (uint32_t*)base.tb, base.skip);
+                       (const V*)a.out, (uint32_t*)base.tb, base.skip);
         else if constexpr (kTensorPhase2x16)
             launch_pdl(k_reduce_pack16_mix, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
                        (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const int32_t*)H.red_order.p,
                        H.n_red_big, H.n_red, (const float*)a.out, (uint16_t*)base.tb, base.skip);
         else if constexpr (NR == 1)
-            launch_pdl(k_reduce_mix<Part, Zt>, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
+            launch_pdl(k_reduce_mix<V, Zt>, dim3(gm), dim3(256), 0, st, (const FarDesc*)H.far.p,
                        (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p, (const int32_t*)H.red_order.p,
                        H.n_red_big, H.n_red,
-                       (const Part*)a.out, (Zt*)base.tb, base.skip);
+                       (const V*)a.out, (Zt*)base.tb, base.skip);
         else
-            launch_pdl(k_reduce_tb<Part, Zt, MODE == 0>, dim3((unsigned)H.n_far), dim3(128), 0, st,
+            launch_pdl(k_reduce_tb<V, Zt, MODE == 0>, dim3((unsigned)H.n_far), dim3(128), 0, st,
                        (const FarDesc*)H.far.p, (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p,
-                       (const Part*)a.out, (Zt*)base.tb, NR, base.skip);
+                       (const V*)a.out, (Zt*)base.tb, NR, base.skip);
         HM_LAUNCH_CHECK();
         if (timed) mark(H, 3, st);
     } else if (timed) {
@@ -2023,9 +2031,7 @@ void ensure_product_scratch(HMat& H, int nrhs, cudaStream_t st) {
     const size_t np = (size_t)std::max<int64_t>(H.p_len, 1) * cap + VEC_SLACK;
     const size_t nt = (size_t)std::max<int64_t>(H.tb_len, 1) * cap + VEC_SLACK;
     H.xc.alloc(nv);
-    H.yc.alloc(nv);
     H.xcf.alloc(nv);
-    H.ycf.alloc(nv);
     H.P.alloc(np);
     H.tb.alloc(nt);
     H.Pf.alloc(np);
