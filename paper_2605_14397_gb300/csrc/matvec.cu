@@ -888,9 +888,9 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
 
     // entry r of the leaf in an output vector (matvec's y in user order: the permutation costs
     // the flush a cached load, a kernel of its own over y cost 3 to 6 us a product)
-    auto out_at = [&](int k, int r) -> Vv& {
-        const int64_t p = (int64_t)L.begin + r / 3;
-        return yc[(int64_t)k * a.ndof + 3 * (a.perm ? (int64_t)a.perm[p] : p) + r % 3];
+    auto out_at = [&](int k, int r) {
+        const int p = L.begin + r / 3;
+        return (int64_t)k * a.ndof + 3 * (int64_t)(a.perm ? __ldg(a.perm + p) : p) + r % 3;
     };
     auto flush = [&]() {
         const LeafSplit sp = a.split[cur];
@@ -928,14 +928,12 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
             for (int e = threadIdx.x; e < KP * rows; e += NCW * 32) {
                 const int kk = e / rows, r = e - kk * rows, k = k0 + kk;
                 if (k >= a.nout) continue;
+                const int64_t dst = whole ? out_at(k, r) : (slot * NR + k) * a.ld_max + r;  // (loads before the sum)
                 const Acc* rk = red + (size_t)kk * NG * (32 * RPL);
                 Acc s = rk[r];
                 for (int q = 1; q < NG; ++q) acc_add(s, rk[(size_t)q * (32 * RPL) + r]);
                 if constexpr (TC16) acc_add(s, ty[(size_t)k * TY_LD + r]);
-                if (whole)
-                    out_at(k, r) = (Vv)acc_value(s);
-                else
-                    slots[(slot * NR + k) * a.ld_max + r] = (Vv)acc_value(s);
+                (whole ? yc : slots)[dst] = (Vv)acc_value(s);
             }
             consumer_sync(NCW * 32);
         }
@@ -954,7 +952,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
                         Vv s = 0;
                         for (int p = 0; p < sp.nparts; ++p)
                             s += __ldcg(slots + ((int64_t)(sp.slot_base + p) * NR + k) * a.ld_max + r);
-                        out_at(k, r) = s;
+                        yc[out_at(k, r)] = s;
                     }
                 if (threadIdx.x == 0) a.counters[cur] = 0;
             }
@@ -1415,6 +1413,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_mr(StreamArgs a) {
 // 65 us at the copy bandwidth): 116 us with scalar operations over 192 rows, 104 us packed
 // over the leaf's row blocks, 92 us with the columns dealt across chunks (deal_start); the
 // whole product 358 us before, 309 now.
+// The sums of up to eight passes, a lane of every eight holding each.
 struct HeldParts {
     FF v;
     int64_t at;  // entry of P; -1: none
@@ -1791,7 +1790,13 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     a.chunks = PL.ch2.p;
     a.cta_begin = PL.cta2.p;
     a.split = PL.split.p;
-    launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST>, dim3(H.grid), dim3((NCW2 + 1) * 32), smem2, st, a);
+    if (H.n_far > 0 && H.p_len > 0) {
+        launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST>, dim3(H.grid), dim3((NCW2 + 1) * 32), smem2, st, a);
+    } else {
+        // without a far field the kernel before is the one that writes x: phase 2 reads x from
+        // its first chunk on and must not start beside it
+        k_phase2<MODE, C, NR, RPL, NCW2, RS, ST><<<H.grid, (NCW2 + 1) * 32, smem2, st>>>(a);
+    }
     HM_LAUNCH_CHECK();
     if (timed) mark(H, 4, st);
 }

@@ -70,3 +70,24 @@ def test_f32_counts_match_f64_vectors(leaf, storage):
         err = np.linalg.norm((y.double() - ref[:nrhs]).cpu().numpy(), axis=1) / scale[:nrhs]
         assert err.max() <= 1e-5, (nrhs, err)
     H.check()
+
+
+def test_near_field_only_products_follow_their_operand():
+    """An operator without admissible blocks: phase 2 comes straight after the kernel that writes
+    its operand.  500 products of changing vectors, each within (eps + 1e-6) of the oracle's."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    el = synth.disk_mesh(24)
+    H = hmat.HMatrix(hmat.ClusterTree(el, 64, 1e-3), el, E, NU, 1e-6, "f32")
+    assert H.info()["u_entries"] == 0
+    A = torch.from_numpy(O.dense_matrix(el, E, NU)).cuda()
+    g = torch.Generator(device="cuda").manual_seed(9)
+    for dt, nrhs in ((torch.float32, 1), (torch.float64, 1), (torch.float32, 3)):
+        xs = torch.randn((500, nrhs, 3 * el.N), generator=g, device="cuda", dtype=dt)
+        ys = torch.empty_like(xs)
+        for q in range(500):
+            H.matvec(xs[q], ys[q])
+        ref = xs.double() @ A.T
+        err = (ys.double() - ref).norm(dim=2) / ref.norm(dim=2)
+        assert err.max().item() <= 2e-6, (dt, nrhs, err.max().item())
