@@ -42,6 +42,7 @@ constexpr int BAR_BYTES = 128;
 // zeroed bytes after phase 1's ring: a single-RHS column read of up to 32 * 12 rows of
 // 4 bytes that starts in the last stage ends inside them
 constexpr int P1_TAIL = 2048;
+constexpr int MAX_RPL = 12;          // 32-row blocks of the largest leaves (384 rows)
 constexpr int VEC_SLACK = 32;        // elements after xc / tb so rounded-up copies stay inside
 
 struct FF {
@@ -1725,8 +1726,12 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
         else
             return k_phase1_f64<C, NR, RPL, NCW>;
     }();
-    const size_t smem1 = BAR_BYTES + (size_t)(MR1 ? MR_STAGES : ST) * STAGE_BYTES + P1_TAIL +
-                         (MR1 ? (size_t)32 * RPL * NR * sizeof(float) : 0);
+    constexpr size_t smem1_ring = BAR_BYTES + (size_t)(MR1 ? MR_STAGES : ST) * STAGE_BYTES + P1_TAIL;
+    constexpr size_t smem1 = smem1_ring + (MR1 ? (size_t)32 * RPL * NR * sizeof(float) : 0);
+    // k_phase1_mr is one function for every RPL: its opt-in is that of the largest leaves,
+    // whichever instantiation of this one sets it (a smaller one set later would refuse them)
+    constexpr size_t smem1_max = smem1_ring + (MR1 ? (size_t)32 * MAX_RPL * NR * sizeof(float) : 0);
+    static_assert(RPL <= MAX_RPL, "the opt-in covers every leaf size");
     // BF16 factors with one RHS: the U slices of phase 2 on tensor cores, which read t in
     // packed BF16 (hi, lo) form (phase 1 stays on the CUDA cores: one mma.sync per 16 x 16
     // tile did not keep up with the stream there)
@@ -1744,7 +1749,7 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     int dev = 0;
     HM_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        HM_CUDA(cudaFuncSetAttribute(phase1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
+        HM_CUDA(cudaFuncSetAttribute(phase1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1_max));
         HM_CUDA(cudaFuncSetAttribute(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
@@ -1814,7 +1819,7 @@ void launch_rpl(HMat& H, const HMat::Plan& PL, const StreamArgs& a, bool timed, 
     } else if (H.ld_max <= 192)
         launch_phases<MODE, C, NR, 6>(H, PL, a, timed, st);
     else
-        launch_phases<MODE, C, NR, 12>(H, PL, a, timed, st);
+        launch_phases<MODE, C, NR, MAX_RPL>(H, PL, a, timed, st);
 }
 
 // The single-RHS FP32-vector product with the ring depth and consumer-warp count of the
