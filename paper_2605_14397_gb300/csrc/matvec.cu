@@ -829,7 +829,7 @@ __device__ __forceinline__ void mr_columns_n(float2 (&t)[RPW][NR / 2], int nact,
 // that packed form), so d(col 0) + d(col 1) = U t for 16 rows.  Warp w = (kg, mg) takes
 // the k-tiles kg, kg + 4 of each slice and keeps m-tiles mg, mg + 4, mg + 8 of the leaf
 // in registers; at the flush each warp adds them to its own row of the reduction buffer.
-template <int MODE, class C, int NR, int RPL, int NCW, int RS, int ST = STAGES>
+template <int MODE, class C, int NR, int RPL, int NCW, int RS, int ST = STAGES, bool TC = true>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     constexpr bool TC2 = MODE == 0 && NR == 1 && RS == 1 && NCW == 16 && RPL == 6 &&
                          std::is_same<C, uint16_t>::value;
@@ -838,7 +838,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     // in TC2, B = t in the packed BF16 (hi, lo) form of k_reduce_pack16_mix read with
     // ldmatrix.trans, two mma per k-tile in two chains.  The CUDA-core accumulators keep the
     // near tiles; the tensor-core results join them at the flush through ty.
-    constexpr bool TC16 = MODE == 0 && NR == 16 && RS == 2 && NCW == 16 && RPL <= 6 &&
+    constexpr bool TC16 = TC && MODE == 0 && NR == 16 && RS == 2 && NCW == 16 && RPL <= 6 &&
                           std::is_same<C, uint16_t>::value;
     constexpr int TC16_MT = 2 * RPL, TY_LD = 196;  // m-tiles of 16 rows; ty row stride (bank spread)
     constexpr int TKG = 4, TMG = 4, TMT = 3;  // k-groups x m-groups = NCW; m-tiles per warp
@@ -1706,7 +1706,7 @@ constexpr int ncw2_for(int NR, int RS) {
     return MODE == 1 && NR > 2 ? 16 - RS : 16;
 }
 
-template <int MODE, class C, int NR, int RPL, int ST = STAGES, int NCW1V = 0, int NCW2V = 0>
+template <int MODE, class C, int NR, int RPL, int ST = STAGES, int NCW1V = 0, int NCW2V = 0, bool TC = true>
 void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool timed, cudaStream_t st) {
     constexpr int NCW = NCW1V ? NCW1V : (MODE == 0 && NR == 16 ? 8 : 16), RS = rs_for<MODE>(NR, RPL),
                   NCW2 = NCW2V ? NCW2V : ncw2_for<MODE>(NR, RS);
@@ -1714,7 +1714,7 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     using Acc = typename AccT<MODE>::type;
     using V = typename AccT<MODE>::vec;
     // BF16 factors with 16 RHS on leaves of up to 192 rows: phase 1 on tensor cores
-    constexpr bool kTensorPhase1 = MODE == 0 && NR == 16 && std::is_same<C, uint16_t>::value && RPL <= 6;
+    constexpr bool kTensorPhase1 = TC && MODE == 0 && NR == 16 && std::is_same<C, uint16_t>::value && RPL <= 6;
     constexpr bool MR1 = MODE == 0 && NR > 4 && !kTensorPhase1;  // phase 1 over column groups
     auto* const phase1 = [] {
         if constexpr (kTensorPhase1)
@@ -1740,7 +1740,7 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
                   "the single-RHS tensor-core phase 2 assumes 16 consumer warps without row split");
     // BF16 factors with 16 RHS: the U slices of phase 2 on tensor cores as well, reading t
     // in the packed BF16 form of k_reduce_pack16_mix
-    constexpr bool kTensorPhase2x16 = MODE == 0 && NR == 16 && std::is_same<C, uint16_t>::value && RPL <= 6;
+    constexpr bool kTensorPhase2x16 = kTensorPhase1;
     constexpr int KP = (MODE == 0 && NR == 16 && RPL <= 6) ? 8 : 1;  // RHS per flush pass of k_phase2
     const size_t smem2 = BAR_BYTES + (size_t)ST * (ZRange<V, NR>::BYTES + STAGE_BYTES) +
                          (size_t)KP * (NCW2 / RS) * 32 * RPL * sizeof(Acc) + (kTensorPhase2x16 ? 16 * 196 * 4 : 0);
@@ -1750,7 +1750,7 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     HM_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
         HM_CUDA(cudaFuncSetAttribute(phase1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1_max));
-        HM_CUDA(cudaFuncSetAttribute(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST>,
+        HM_CUDA(cudaFuncSetAttribute(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }
@@ -1796,17 +1796,17 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     a.cta_begin = PL.cta2.p;
     a.split = PL.split.p;
     if (H.n_far > 0 && H.p_len > 0) {
-        launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST>, dim3(H.grid), dim3((NCW2 + 1) * 32), smem2, st, a);
+        launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC>, dim3(H.grid), dim3((NCW2 + 1) * 32), smem2, st, a);
     } else {
         // without a far field the kernel before is the one that writes x: phase 2 reads x from
         // its first chunk on and must not start beside it
-        k_phase2<MODE, C, NR, RPL, NCW2, RS, ST><<<H.grid, (NCW2 + 1) * 32, smem2, st>>>(a);
+        k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC><<<H.grid, (NCW2 + 1) * 32, smem2, st>>>(a);
     }
     HM_LAUNCH_CHECK();
     if (timed) mark(H, 4, st);
 }
 
-template <int MODE, class C, int NR>
+template <int MODE, class C, int NR, bool TC = true>
 void launch_rpl(HMat& H, const HMat::Plan& PL, const StreamArgs& a, bool timed, cudaStream_t st) {
     // 16 RHS split a column's rows over two warps, so leaves of at most 128 rows have a
     // variant of their own: with three row blocks a warp, one of 99 rows left the second warp
@@ -1815,9 +1815,9 @@ void launch_rpl(HMat& H, const HMat::Plan& PL, const StreamArgs& a, bool timed, 
     // a split computed from each leaf's rows cost the 176-row leaves of three 100 x 100 planes
     // 10 %)
     if (NR == 16 && H.ld_max <= 128) {
-        if constexpr (NR == 16) launch_phases<MODE, C, NR, 4>(H, PL, a, timed, st);
+        if constexpr (NR == 16) launch_phases<MODE, C, NR, 4, STAGES, 0, 0, TC>(H, PL, a, timed, st);
     } else if (H.ld_max <= 192)
-        launch_phases<MODE, C, NR, 6>(H, PL, a, timed, st);
+        launch_phases<MODE, C, NR, 6, STAGES, 0, 0, TC>(H, PL, a, timed, st);
     else
         launch_phases<MODE, C, NR, MAX_RPL>(H, PL, a, timed, st);
 }
@@ -1856,15 +1856,22 @@ void launch_nr(HMat& H, const HMat::Plan& PL, const StreamArgs& a, int nrhs, boo
             case 1: return launch_rpl<MODE, C, 1>(H, PL, a, timed, st);
             case 4: return launch_rpl<MODE, C, 4>(H, PL, a, timed, st);
             case 8: return launch_rpl<MODE, C, 8>(H, PL, a, timed, st);
-            case 16: return launch_rpl<MODE, C, 16>(H, PL, a, timed, st);
+            case 16:
+                if constexpr (std::is_same<C, uint16_t>::value) {
+                    // The tensor-core phases keep about 16 bits of the vectors, which the
+                    // interface states for full passes only: 9 to 15 keep FP32 vectors
+                    // (12 on three 150 x 150 planes: 1.94 ms; 16 on tensor cores: 1.21).
+                    if (a.nout < 16) return launch_rpl<MODE, C, 16, false>(H, PL, a, timed, st);
+                }
+                return launch_rpl<MODE, C, 16>(H, PL, a, timed, st);
             default: fail(HM_EINVAL, "product: 1, 4, 8 or 16 right-hand sides per F32 pass");
         }
     }
 }
 
 // The F32 kernels take 1, 4, 8 or 16 right-hand sides: other counts are padded with zero
-// vectors, whose products are not written.  (The kernels that tested each count in their
-// loops took 3.18 ms for 12 BF16 right-hand sides on three 150 x 150 planes, 1.44 ms for 16.)
+// vectors, whose products are not written.  (12 right-hand sides, BF16 factors, three 150 x
+// 150 planes: 4.03 ms with kernels that tested the count in their loops, 1.94 padded.)
 int padded_rhs(int nr) { return nr == 1 ? 1 : (nr <= 4 ? 4 : (nr <= 8 ? 8 : 16)); }
 
 // phase 1, reduction and phase 2 on cluster-ordered operands (see hmat_impl.h); F32: xc
