@@ -635,6 +635,15 @@ struct StreamArgs {
     int64_t withhold;
 };
 
+// True when every right-hand side has converged: the kernel has nothing to do.  It still waits
+// for the kernel before it, which may have let it start early: the next launch is ordered
+// after this kernel only.
+__device__ __forceinline__ bool skipped(const StreamArgs& a) {
+    if (!a.skip || !*(volatile const int*)a.skip) return false;
+    pdl_wait();
+    return true;
+}
+
 template <class V, int NR>
 struct ZRange {
     static constexpr int ALIGN = 16 / (int)sizeof(V);  // elements per 16 bytes
@@ -865,7 +874,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     Acc* red = (Acc*)(stage + (size_t)ST * STRIDE);  // [KP][NG][32 RPL]
     float* ty = (float*)(red + (size_t)KP * NG * 32 * RPL);  // TC16: the leaf's tensor-core sums [16 RHS][TY_LD]
 
-    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
+    if (skipped(a)) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x < 8) zline[threadIdx.x] = 0;
     init_ring<ST>(full, empty, NCW);
@@ -1128,7 +1137,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
     uint64_t* empty = full + ST;
     unsigned char* stage = smem + BAR_BYTES;
 
-    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
+    if (skipped(a)) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if constexpr (NR == 1) {
         // The single-RHS loop reads whole 32 RPL-row columns without bound checks: rows past
@@ -1290,7 +1299,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_mr(StreamArgs a) {
     uint64_t* empty = full + MR_STAGES;
     unsigned char* stage = smem + BAR_BYTES;
     float4* xs = (float4*)(stage + MR_STAGES * STAGE_BYTES + P1_TAIL);  // the leaf's operands (mr_x_index)
-    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
+    if (skipped(a)) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, cg = lane >> 3, rl = lane & 7;
     {
         uint4* z = reinterpret_cast<uint4*>(stage);
@@ -1483,7 +1492,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_f64(StreamArgs a) 
     uint64_t* full = (uint64_t*)smem;
     uint64_t* empty = full + STAGES;
     unsigned char* stage = smem + BAR_BYTES;
-    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
+    if (skipped(a)) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     {  // finite data behind every unchecked column read, as in k_phase1
         uint4* z = reinterpret_cast<uint4*>(stage);
@@ -1561,7 +1570,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_tc(StreamArgs a) {
     uint64_t* empty = full + STAGES;
     unsigned char* stage = smem + BAR_BYTES;
 
-    if (a.skip && *(volatile const int*)a.skip) return;
+    if (skipped(a)) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     {  // finite data behind every unchecked read, as in k_phase1
         uint4* z = reinterpret_cast<uint4*>(stage);
