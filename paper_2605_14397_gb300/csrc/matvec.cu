@@ -627,6 +627,7 @@ struct StreamArgs {
     int64_t ndof;
     int nout;     // right-hand sides the caller asked for (the vectors of out); the rest pad the kernel's count
     int ld_max;
+    int wait_x;   // phase 2: xc comes from the kernel just before (no far field, so no kernel in between)
     const int* skip;  // optional device flag: when set, the kernels return at once
     uint64_t wait_ns; // limit of every bounded wait of the copy ring
     // test switch (hm_hmat_set_wait): the producer of phase 2 stops before this chunk of
@@ -667,7 +668,8 @@ __device__ __forceinline__ int deal_next(int rot, int n) {
 
 // ---- producer: one thread streams this CTA's chunks (and their operands) through the ring
 // (WAIT_T: wait for the preceding kernel -- the reduction producing t -- only before the
-// first chunk whose operand is t; near tiles read x, complete before that kernel began)
+// first chunk whose operand is t; near tiles read x, complete before that kernel began.
+// Without a far field the preceding kernel is the one that writes x: wait_x.)
 template <class C, class V, int NR, bool WITH_Z, bool WAIT_T = false, int ST = STAGES>
 __device__ __forceinline__ void produce(const StreamArgs& a, unsigned char* smem_stage, int stage_stride,
                                         uint64_t* full, uint64_t* empty, int c0, int c1) {
@@ -683,7 +685,7 @@ __device__ __forceinline__ void produce(const StreamArgs& a, unsigned char* smem
         const Chunk ch = nxt;
         if (i + 1 < c1) nxt = a.chunks[i + 1];
         if constexpr (WAIT_T) {
-            if (!waited && ch.kind != 0) {
+            if (!waited && (ch.kind != 0 || a.wait_x)) {
                 pdl_wait();
                 waited = true;
             }
@@ -1804,13 +1806,8 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     a.chunks = PL.ch2.p;
     a.cta_begin = PL.cta2.p;
     a.split = PL.split.p;
-    if (H.n_far > 0 && H.p_len > 0) {
-        launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC>, dim3(H.grid), dim3((NCW2 + 1) * 32), smem2, st, a);
-    } else {
-        // without a far field the kernel before is the one that writes x: phase 2 reads x from
-        // its first chunk on and must not start beside it
-        k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC><<<H.grid, (NCW2 + 1) * 32, smem2, st>>>(a);
-    }
+    a.wait_x = !(H.n_far > 0 && H.p_len > 0);
+    launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC>, dim3(H.grid), dim3((NCW2 + 1) * 32), smem2, st, a);
     HM_LAUNCH_CHECK();
     if (timed) mark(H, 4, st);
 }
