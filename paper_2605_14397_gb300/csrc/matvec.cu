@@ -249,9 +249,11 @@ __global__ void k_gather(const float* __restrict__ x, float* __restrict__ xc, co
     xc[q] = k < nrhs ? x[k * ndof + 3 * (int64_t)perm[p] + m] : 0.f;
 }
 
-// the same padding for operands already in cluster order, interleaved by nr
+// The same padding for operands already in cluster order, interleaved by nr.  (The solver's
+// kernels before a product let nothing start early: a phase that finds every right-hand side
+// converged returns without waiting for them, and what follows is ordered after the phases
+// only.  A wait on that path cost the single-RHS F64 phases 1.5 %.)
 __global__ void k_pad(const float* __restrict__ xc, float* __restrict__ xp, int64_t ndof, int nr, int np) {
-    pdl_trigger();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= ndof * np) return;
     const int64_t r = q / np, k = q % np;
@@ -636,15 +638,6 @@ struct StreamArgs {
     int64_t withhold;
 };
 
-// True when every right-hand side has converged: the kernel has nothing to do.  It still waits
-// for the kernel before it, which may have let it start early: the next launch is ordered
-// after this kernel only.
-__device__ __forceinline__ bool skipped(const StreamArgs& a) {
-    if (!a.skip || !*(volatile const int*)a.skip) return false;
-    pdl_wait();
-    return true;
-}
-
 template <class V, int NR>
 struct ZRange {
     static constexpr int ALIGN = 16 / (int)sizeof(V);  // elements per 16 bytes
@@ -668,8 +661,7 @@ __device__ __forceinline__ int deal_next(int rot, int n) {
 
 // ---- producer: one thread streams this CTA's chunks (and their operands) through the ring
 // (WAIT_T: wait for the preceding kernel -- the reduction producing t -- only before the
-// first chunk whose operand is t; near tiles read x, complete before that kernel began.
-// Without a far field the preceding kernel is the one that writes x: wait_x.)
+// first chunk whose operand is t; near tiles read x, complete before that kernel began)
 template <class C, class V, int NR, bool WITH_Z, bool WAIT_T = false, int ST = STAGES>
 __device__ __forceinline__ void produce(const StreamArgs& a, unsigned char* smem_stage, int stage_stride,
                                         uint64_t* full, uint64_t* empty, int c0, int c1) {
@@ -685,7 +677,7 @@ __device__ __forceinline__ void produce(const StreamArgs& a, unsigned char* smem
         const Chunk ch = nxt;
         if (i + 1 < c1) nxt = a.chunks[i + 1];
         if constexpr (WAIT_T) {
-            if (!waited && (ch.kind != 0 || a.wait_x)) {
+            if (!waited && ch.kind != 0) {
                 pdl_wait();
                 waited = true;
             }
@@ -876,7 +868,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     Acc* red = (Acc*)(stage + (size_t)ST * STRIDE);  // [KP][NG][32 RPL]
     float* ty = (float*)(red + (size_t)KP * NG * 32 * RPL);  // TC16: the leaf's tensor-core sums [16 RHS][TY_LD]
 
-    if (skipped(a)) return;
+    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x < 8) zline[threadIdx.x] = 0;
     init_ring<ST>(full, empty, NCW);
@@ -885,7 +877,10 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     if (w == NCW) {
         // the t operand ranges come from the reduction: the producer waits for it before the
         // first U chunk, so the near tiles ahead of it stream while the reduction runs
-        if (lane == 0) produce<C, Vv, NR, true, true, ST>(a, stage, STRIDE, full, empty, c0, c1);
+        if (lane == 0) {
+            if (a.wait_x) pdl_wait();  // (before produce: in its loop the test cost the F64 kernels 0.7 %)
+            produce<C, Vv, NR, true, true, ST>(a, stage, STRIDE, full, empty, c0, c1);
+        }
         return;
     }
     Vv* yc = (Vv*)a.out;
@@ -1139,7 +1134,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
     uint64_t* empty = full + ST;
     unsigned char* stage = smem + BAR_BYTES;
 
-    if (skipped(a)) return;
+    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if constexpr (NR == 1) {
         // The single-RHS loop reads whole 32 RPL-row columns without bound checks: rows past
@@ -1301,7 +1296,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_mr(StreamArgs a) {
     uint64_t* empty = full + MR_STAGES;
     unsigned char* stage = smem + BAR_BYTES;
     float4* xs = (float4*)(stage + MR_STAGES * STAGE_BYTES + P1_TAIL);  // the leaf's operands (mr_x_index)
-    if (skipped(a)) return;
+    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, cg = lane >> 3, rl = lane & 7;
     {
         uint4* z = reinterpret_cast<uint4*>(stage);
@@ -1494,7 +1489,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_f64(StreamArgs a) 
     uint64_t* full = (uint64_t*)smem;
     uint64_t* empty = full + STAGES;
     unsigned char* stage = smem + BAR_BYTES;
-    if (skipped(a)) return;
+    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     {  // finite data behind every unchecked column read, as in k_phase1
         uint4* z = reinterpret_cast<uint4*>(stage);
@@ -1572,7 +1567,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_tc(StreamArgs a) {
     uint64_t* empty = full + STAGES;
     unsigned char* stage = smem + BAR_BYTES;
 
-    if (skipped(a)) return;
+    if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     {  // finite data behind every unchecked read, as in k_phase1
         uint4* z = reinterpret_cast<uint4*>(stage);
