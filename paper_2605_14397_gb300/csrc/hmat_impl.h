@@ -212,12 +212,14 @@ void timing_enable(HMat& H, bool on);
 void timing_read(HMat& H, double out[6]);
 void matvec_host(HMat& H, const void* x, void* y, int nrhs, int dtype, cudaStream_t st);
 void matvec(HMat& H, const void* x, void* y, int nrhs, int dtype, cudaStream_t st, int factors = 0);
-// Product on cluster-ordered operands: xc is RHS-interleaved (xc[dof * nr + k]) with at
-// least 32 readable elements after its end, yc is RHS-major (yc[k * ndof + dof]).
-// fac: 0 FP32 factors, 1 BF16 factors.  dtype HM_F32: float vectors; HM_F64: xc holds
-// every double pre-split into (hi, lo) floats (float2, written by the gather or the
-// solver), yc doubles.  At most product_pass(dtype) right-hand sides.
-int product_pass(int dtype);
+// Product on cluster-ordered operands: xc with at least 32 readable elements after its end,
+// yc RHS-major (yc[k * ndof + dof]).  fac: 0 FP32 factors, 1 BF16 factors.  dtype HM_F32:
+// float vectors, xc RHS-interleaved (xc[dof * nr + k]); HM_F64: yc doubles, xc as
+// product_split writes it from the RHS-major doubles z (zs: nr rounded up to a multiple of
+// four vectors, and 8 elements).  Of nr right-hand sides the next product_group(H, nr, dtype)
+// go at once.
+int product_group(const HMat& H, int nr, int dtype);
+void product_split(HMat& H, const double* z, double* zs, int nr, cudaStream_t st);
 void product_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, cudaStream_t st,
                   const int* skip = nullptr);
 // Concatenate independent H-matrices into one (block-diagonal operator, one work list).

@@ -56,7 +56,7 @@ struct FF2 {
 // right-hand side, so from four on the pass is bound by the FP32 pipe and streaming the
 // coefficients again for the next four costs less than the registers of a wider pass:
 // six RHS of a 12,892-element fault (615 MB of coefficients) took 2.82 ms in one pass of a
-// 16-wide kernel that spilled, 0.60 ms in passes of four and two.
+// 16-wide kernel that spilled, 0.56 ms in two passes of three (f64_passes).
 constexpr int F64_PASS = 4;
 
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -260,16 +260,18 @@ __global__ void k_pad(const float* __restrict__ xc, float* __restrict__ xp, int6
     xp[q] = k < nr ? xc[r * nr + k] : 0.f;
 }
 
-// F64 gather: xc[dof * nr + k] = (hi, lo) split of x[k * ndof + user dof]
+// F64 gather: xc[pass * xc_pass + dof * width + k] = (hi, lo) split of x[(pass * width + k) * ndof +
+// user dof], zero beyond nrhs; perm NULL: x is in cluster order already (a solver's: as k_pad)
 __global__ void k_gather_split(const double* __restrict__ x, float2* __restrict__ xc,
-                               const int32_t* __restrict__ perm, int64_t N, int nrhs) {
-    pdl_trigger();
+                               const int32_t* __restrict__ perm, int64_t N, int nrhs, int width, int64_t xc_pass) {
+    if (perm) pdl_trigger();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t ndof = 3 * N;
-    if (q >= ndof * nrhs) return;
-    const int64_t r = q / nrhs, k = q % nrhs;
+    if (q >= ndof * width) return;
+    const int64_t r = q / width, k = blockIdx.y * (int64_t)width + q % width;
     const int64_t p = r / 3, m = r % 3;
-    xc[q] = split_d(x[k * ndof + 3 * (int64_t)perm[p] + m]);
+    xc[blockIdx.y * xc_pass + q] =
+        k < nrhs ? split_d(x[k * ndof + 3 * (perm ? (int64_t)perm[p] : p) + m]) : make_float2(0.f, 0.f);
 }
 
 __device__ __forceinline__ float to_zin(float v, float*) { return v; }
@@ -283,14 +285,16 @@ __device__ __forceinline__ uint32_t to_zin(float v, uint32_t*) {
 
 // tb[(tb_off + l) nr + k] = sum_q P[(poff[pbase + q] + l) nr + k], one CTA (128 threads)
 // (VEC4: FP32 with nr a multiple of 4, each slice read as float4)
-// per block: the n = r nr entries times G = 128 / n interleaved groups of leaf partials,
+// per block (and F64 pass): the n = r nr entries times G = 128 / n interleaved groups of leaf partials,
 // four independent loads in flight per thread, groups combined in a fixed order.  In F64
 // mode the sums are stored as (hi, lo) float pairs, the form phase 2 reads.
 template <class V, class Zt, bool VEC4>
 __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ far, const int32_t* __restrict__ poff,
                                                    const int32_t* __restrict__ uoff, const V* __restrict__ P,
-                                                   Zt* __restrict__ tb, int nrhs, const int* __restrict__ skip) {
+                                                   Zt* __restrict__ tb, int nrhs, int64_t p_pass, int64_t tb_pass,
+                                                   const int* __restrict__ skip) {
     __shared__ V sp[128];
+    const int64_t p0 = VEC4 ? 0 : blockIdx.y * p_pass, t0 = VEC4 ? 0 : blockIdx.y * tb_pass;
     pdl_wait();
     pdl_trigger();
     if (skip && *(volatile const int*)skip) return;
@@ -307,7 +311,7 @@ __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ f
         __syncthreads();
         po = spo;
     }
-    auto at = [&](int q) -> int64_t { return (int64_t)po[q] * nrhs; };
+    auto at = [&](int q) -> int64_t { return p0 + (int64_t)po[q] * nrhs; };
     if constexpr (VEC4) {
         {
             // several RHS: each slice is rank * nrhs contiguous floats, read as float4
@@ -353,7 +357,7 @@ __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ f
             }
             for (; q < F.n_tleaves; ++q) s0 += P[at(q) + e];
             const Zt t = to_zin((s0 + s1) + (s2 + s3), tb);
-            for (int c = 0; c < F.n_sleaves; ++c) tb[(int64_t)uoff[F.ubase + c] * nrhs + e] = t;
+            for (int c = 0; c < F.n_sleaves; ++c) tb[t0 + (int64_t)uoff[F.ubase + c] * nrhs + e] = t;
         }
         return;
     }
@@ -376,7 +380,7 @@ __global__ void __launch_bounds__(128) k_reduce_tb(const FarDesc* __restrict__ f
         V s = 0;
         for (int q = 0; q < G; ++q) s += sp[q * n + threadIdx.x];
         const Zt t = to_zin(s, tb);
-        for (int c = 0; c < F.n_sleaves; ++c) tb[(int64_t)uoff[F.ubase + c] * nrhs + threadIdx.x] = t;
+        for (int c = 0; c < F.n_sleaves; ++c) tb[t0 + (int64_t)uoff[F.ubase + c] * nrhs + threadIdx.x] = t;
     }
 }
 
@@ -629,6 +633,10 @@ struct StreamArgs {
     int64_t ndof;
     int nout;     // right-hand sides the caller asked for (the vectors of out); the rest pad the kernel's count
     int ld_max;
+    // F64: more right-hand sides than one pass holds run as passes of NR in the same launches
+    // (blockIdx.y).  Elements from one pass's xc, P and tb to the next's, and its slots and counters
+    int64_t xc_pass, p_pass, tb_pass;
+    int slots_pass, counters_pass;
     int wait_x;   // phase 2: xc comes from the kernel just before (no far field, so no kernel in between)
     const int* skip;  // optional device flag: when set, the kernels return at once
     uint64_t wait_ns; // limit of every bounded wait of the copy ring
@@ -832,8 +840,9 @@ __device__ __forceinline__ void mr_columns_n(float2 (&t)[RPW][NR / 2], int nact,
 // that packed form), so d(col 0) + d(col 1) = U t for 16 rows.  Warp w = (kg, mg) takes
 // the k-tiles kg, kg + 4 of each slice and keeps m-tiles mg, mg + 4, mg + 8 of the leaf
 // in registers; at the flush each warp adds them to its own row of the reduction buffer.
-template <int MODE, class C, int NR, int RPL, int NCW, int RS, int ST = STAGES, bool TC = true>
+template <int MODE, class C, int NR, int RPL, int NCW, int RS, int ST = STAGES, bool TC = true, bool PASSES = false>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
+    static_assert(!PASSES || MODE == 1, "F64 passes");
     constexpr bool TC2 = MODE == 0 && NR == 1 && RS == 1 && NCW == 16 && RPL == 6 &&
                          std::is_same<C, uint16_t>::value;
     // BF16 U slices with 16 RHS (TC16): warp w owns the m-tiles w / 2 and w / 2 + 8 (16 rows
@@ -877,6 +886,10 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     if (w == NCW) {
         // the t operand ranges come from the reduction: the producer waits for it before the
         // first U chunk, so the near tiles ahead of it stream while the reduction runs
+        if constexpr (PASSES) {
+            a.xc = (const Vv*)a.xc + blockIdx.y * a.xc_pass;
+            a.tb = (const Vv*)a.tb + blockIdx.y * a.tb_pass;
+        }
         if (lane == 0) {
             if (a.wait_x) pdl_wait();  // (before produce: in its loop the test cost the F64 kernels 0.7 %)
             produce<C, Vv, NR, true, true, ST>(a, stage, STRIDE, full, empty, c0, c1);
@@ -885,6 +898,14 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     }
     Vv* yc = (Vv*)a.out;
     Vv* slots = (Vv*)a.slots;
+    int nout = a.nout;
+    int32_t* counters = a.counters;
+    if constexpr (PASSES) {
+        nout = min(NR, a.nout - (int)blockIdx.y * NR);
+        yc += (int64_t)blockIdx.y * NR * a.ndof;
+        slots += (int64_t)blockIdx.y * a.slots_pass * NR * a.ld_max;
+        counters += blockIdx.y * a.counters_pass;
+    }
     const int g = w / RS, rbase = (w % RS) * 32 * RPW;
     constexpr bool MR = MODE == 0 && NR > 1;  // accumulators in RHS pairs
     Acc acc[MR ? 1 : NR][RPW];
@@ -908,7 +929,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
         // runtime index into acc would move it to local memory)
 #pragma unroll
         for (int k0 = 0; k0 < NR; k0 += KP) {
-            if (k0 >= a.nout) break;
+            if (k0 >= nout) break;
 #pragma unroll
             for (int kk = 0; kk < KP; ++kk)
 #pragma unroll
@@ -934,7 +955,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
             consumer_sync(NCW * 32);
             for (int e = threadIdx.x; e < KP * rows; e += NCW * 32) {
                 const int kk = e / rows, r = e - kk * rows, k = k0 + kk;
-                if (k >= a.nout) continue;
+                if (k >= nout) continue;
                 const int64_t dst = whole ? out_at(k, r) : (slot * NR + k) * a.ld_max + r;  // (loads before the sum)
                 const Acc* rk = red + (size_t)kk * NG * (32 * RPL);
                 Acc s = rk[r];
@@ -948,20 +969,20 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
             __threadfence();
             consumer_sync(NCW * 32);
             if (threadIdx.x == 0) {
-                const int old = atomicAdd(a.counters + cur, 1);
+                const int old = atomicAdd(counters + cur, 1);
                 *s_flag = (old == sp.nparts - 1);
             }
             consumer_sync(NCW * 32);
             if (*s_flag) {
                 __threadfence();
-                for (int k = 0; k < a.nout; ++k)
+                for (int k = 0; k < nout; ++k)
                     for (int r = threadIdx.x; r < rows; r += NCW * 32) {
                         Vv s = 0;
                         for (int p = 0; p < sp.nparts; ++p)
                             s += __ldcg(slots + ((int64_t)(sp.slot_base + p) * NR + k) * a.ld_max + r);
                         yc[out_at(k, r)] = s;
                     }
-                if (threadIdx.x == 0) a.counters[cur] = 0;
+                if (threadIdx.x == 0) counters[cur] = 0;
             }
             consumer_sync(NCW * 32);
         }
@@ -1483,13 +1504,16 @@ __device__ __forceinline__ void ff_phase1_columns(const float2 (&x)[NR][RPL], co
     }
 }
 
-template <class C, int NR, int RPL, int NCW>
+template <class C, int NR, int RPL, int NCW, bool PASSES>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_f64(StreamArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t* full = (uint64_t*)smem;
     uint64_t* empty = full + STAGES;
     unsigned char* stage = smem + BAR_BYTES;
     if (a.skip && *(volatile const int*)a.skip) return;  // every right-hand side already converged
+    if constexpr (PASSES) {  // fewer chunks than CTAs: the next pass's CTA takes the SM
+        if (a.cta_begin[blockIdx.x] == a.cta_begin[blockIdx.x + 1]) return;
+    }
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     {  // finite data behind every unchecked column read, as in k_phase1
         uint4* z = reinterpret_cast<uint4*>(stage);
@@ -1507,8 +1531,12 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1_f64(StreamArgs a) 
     }
     pdl_wait();  // x in cluster order comes from the preceding kernel
     double* P = (double*)a.out;
-    HeldParts held{FF{0.f, 0.f}, -1, 0};
     const float2* xs = (const float2*)a.xc;
+    if constexpr (PASSES) {
+        P += blockIdx.y * a.p_pass;
+        xs += blockIdx.y * a.xc_pass;
+    }
+    HeldParts held{FF{0.f, 0.f}, -1, 0};
     int cur = -1, rows = 0, rot = 0;
     float2 x[NR][RPL];
     auto load = [lane](const C* col, int i) { return coef(col, lane + 32 * i); };
@@ -1712,7 +1740,8 @@ constexpr int ncw2_for(int NR, int RS) {
     return MODE == 1 && NR > 2 ? 16 - RS : 16;
 }
 
-template <int MODE, class C, int NR, int RPL, int ST = STAGES, int NCW1V = 0, int NCW2V = 0, bool TC = true>
+template <int MODE, class C, int NR, int RPL, int ST = STAGES, int NCW1V = 0, int NCW2V = 0, bool TC = true,
+          bool PASSES = false>
 void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool timed, cudaStream_t st) {
     constexpr int NCW = NCW1V ? NCW1V : (MODE == 0 && NR == 16 ? 8 : 16), RS = rs_for<MODE>(NR, RPL),
                   NCW2 = NCW2V ? NCW2V : ncw2_for<MODE>(NR, RS);
@@ -1730,7 +1759,7 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
         else if constexpr (MODE == 0)
             return k_phase1<C, NR, RPL, NCW, ST>;
         else
-            return k_phase1_f64<C, NR, RPL, NCW>;
+            return k_phase1_f64<C, NR, RPL, NCW, PASSES>;
     }();
     constexpr size_t smem1_ring = BAR_BYTES + (size_t)(MR1 ? MR_STAGES : ST) * STAGE_BYTES + P1_TAIL;
     constexpr size_t smem1 = smem1_ring + (MR1 ? (size_t)32 * RPL * NR * sizeof(float) : 0);
@@ -1756,16 +1785,17 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     HM_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
         HM_CUDA(cudaFuncSetAttribute(phase1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1_max));
-        HM_CUDA(cudaFuncSetAttribute(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC>,
+        HM_CUDA(cudaFuncSetAttribute(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC, PASSES>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }
+    const unsigned passes = PASSES ? (unsigned)ceil_div(base.nout, NR) : 1u;
     if (H.n_far > 0 && H.p_len > 0) {
         StreamArgs a = base;
         a.chunks = PL.ch1.p;
         a.cta_begin = PL.cta1.p;
         a.out = MODE == 0 ? (void*)H.Pf.p : (void*)H.P.p;
-        launch_pdl(phase1, dim3(H.grid), dim3((NCW + 1) * 32), smem1, st, a);
+        launch_pdl(phase1, dim3(H.grid, passes), dim3((NCW + 1) * 32), smem1, st, a);
         HM_LAUNCH_CHECK();
         if (timed) mark(H, 2, st);
         using Zt = typename AccT<MODE>::zin;
@@ -1788,9 +1818,9 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
                        H.n_red_big, H.n_red,
                        (const V*)a.out, (Zt*)base.tb, base.skip);
         else
-            launch_pdl(k_reduce_tb<V, Zt, MODE == 0>, dim3((unsigned)H.n_far), dim3(128), 0, st,
+            launch_pdl(k_reduce_tb<V, Zt, MODE == 0>, dim3((unsigned)H.n_far, passes), dim3(128), 0, st,
                        (const FarDesc*)H.far.p, (const int32_t*)H.poff.p, (const int32_t*)H.uoff.p,
-                       (const V*)a.out, (Zt*)base.tb, NR, base.skip);
+                       (const V*)a.out, (Zt*)base.tb, NR, base.p_pass, base.tb_pass, base.skip);
         HM_LAUNCH_CHECK();
         if (timed) mark(H, 3, st);
     } else if (timed) {
@@ -1802,12 +1832,12 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     a.cta_begin = PL.cta2.p;
     a.split = PL.split.p;
     a.wait_x = !(H.n_far > 0 && H.p_len > 0);
-    launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC>, dim3(H.grid), dim3((NCW2 + 1) * 32), smem2, st, a);
+    launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC, PASSES>, dim3(H.grid, passes), dim3((NCW2 + 1) * 32), smem2, st, a);
     HM_LAUNCH_CHECK();
     if (timed) mark(H, 4, st);
 }
 
-template <int MODE, class C, int NR, bool TC = true>
+template <int MODE, class C, int NR, bool TC = true, bool PASSES = false>
 void launch_rpl(HMat& H, const HMat::Plan& PL, const StreamArgs& a, bool timed, cudaStream_t st) {
     // 16 RHS split a column's rows over two warps, so leaves of at most 128 rows have a
     // variant of their own: with three row blocks a warp, one of 99 rows left the second warp
@@ -1816,11 +1846,11 @@ void launch_rpl(HMat& H, const HMat::Plan& PL, const StreamArgs& a, bool timed, 
     // a split computed from each leaf's rows cost the 176-row leaves of three 100 x 100 planes
     // 10 %)
     if (NR == 16 && H.ld_max <= 128) {
-        if constexpr (NR == 16) launch_phases<MODE, C, NR, 4, STAGES, 0, 0, TC>(H, PL, a, timed, st);
+        if constexpr (NR == 16) launch_phases<MODE, C, NR, 4, STAGES, 0, 0, TC, PASSES>(H, PL, a, timed, st);
     } else if (H.ld_max <= 192)
-        launch_phases<MODE, C, NR, 6, STAGES, 0, 0, TC>(H, PL, a, timed, st);
+        launch_phases<MODE, C, NR, 6, STAGES, 0, 0, TC, PASSES>(H, PL, a, timed, st);
     else
-        launch_phases<MODE, C, NR, MAX_RPL>(H, PL, a, timed, st);
+        launch_phases<MODE, C, NR, MAX_RPL, STAGES, 0, 0, true, PASSES>(H, PL, a, timed, st);
 }
 
 // The single-RHS FP32-vector product with the ring depth and consumer-warp count of the
@@ -1845,12 +1875,16 @@ bool launch_shape_variant(HMat& H, const HMat::Plan& PL, const StreamArgs& a, bo
 template <int MODE, class C>
 void launch_nr(HMat& H, const HMat::Plan& PL, const StreamArgs& a, int nrhs, bool timed, cudaStream_t st) {
     if constexpr (MODE == 1) {
+        if (a.nout > nrhs) {  // several passes: of three or four
+            return nrhs == 3 ? launch_rpl<MODE, C, 3, true, true>(H, PL, a, timed, st)
+                             : launch_rpl<MODE, C, 4, true, true>(H, PL, a, timed, st);
+        }
         switch (nrhs) {
             case 1: return launch_rpl<MODE, C, 1>(H, PL, a, timed, st);
             case 2: return launch_rpl<MODE, C, 2>(H, PL, a, timed, st);
             case 3: return launch_rpl<MODE, C, 3>(H, PL, a, timed, st);
             case 4: return launch_rpl<MODE, C, 4>(H, PL, a, timed, st);
-            default: fail(HM_EINVAL, "product: 1 to 4 right-hand sides per F64 pass");
+            default: fail(HM_EINVAL, "product: F64 passes of 1 to 4 right-hand sides");
         }
     } else {
         switch (nrhs) {
@@ -1875,8 +1909,29 @@ void launch_nr(HMat& H, const HMat::Plan& PL, const StreamArgs& a, int nrhs, boo
 // 150 planes: 4.03 ms with kernels that tested the count in their loops, 1.94 padded.)
 int padded_rhs(int nr) { return nr == 1 ? 1 : (nr <= 4 ? 4 : (nr <= 8 ? 8 : 16)); }
 
+// The F64 passes that share one set of launches for the first right-hand sides of nr: count of
+// them, width of each, right-hand sides covered.  A set of launches costs 12 to 15 us where the
+// operator is small: 16 right-hand sides of 256 elements took 90 us in four sets, 58 us in the
+// single wide pass those had replaced, and take 31 us as four passes of one set; 12,892
+// elements: 1,457 us in four sets, 1,401 us in one.  Where nr does not divide, equal passes are
+// padded with zero vectors as long as the work of those (F64_PAD_COEFS stored coefficients,
+// about 5 us) is below a set of launches; beyond, the passes of four go first and the rest is a
+// set of its own.
+struct F64Passes {
+    int count, width, nrhs;
+};
+constexpr int64_t F64_PAD_COEFS = 16 << 20;
+F64Passes f64_passes(const HMat& H, int nr) {
+    nr = std::min(nr, 16);
+    const int count = (int)ceil_div(nr, F64_PASS), width = (int)ceil_div(nr, count);
+    if ((count * width - nr) * (H.near_entries + H.far_entries) <= F64_PAD_COEFS) return F64Passes{count, width, nr};
+    return F64Passes{nr / F64_PASS, F64_PASS, nr / F64_PASS * F64_PASS};
+}
+// elements of one pass's interleaved vectors of len entries: the next pass starts 16-byte aligned
+int64_t f64_pass_stride(int64_t len, int width) { return (len * width + 1) & ~(int64_t)1; }
+
 // phase 1, reduction and phase 2 on cluster-ordered operands (see hmat_impl.h); F32: xc
-// interleaved by padded_rhs(nr).  perm: yc in user order.
+// interleaved by padded_rhs(nr); F64: as k_gather_split lays it out for f64_passes(nr).  perm: yc in user order.
 void run_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, bool timed, cudaStream_t st,
               const int* skip = nullptr, const int32_t* perm = nullptr) {
     if (!has_factors(H, fac)) fail(HM_EINVAL, "product: the requested factor precision is not stored");
@@ -1910,10 +1965,17 @@ void run_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, boo
     } else {
         a.tb = H.tb.p;
         a.slots = H.slotsd.p;
+        const F64Passes ps = f64_passes(H, nr);
+        if (ps.nrhs != nr) fail(HM_EINVAL, "product: right-hand sides of more than one set of F64 passes");
+        a.xc_pass = f64_pass_stride(H.ndof, ps.width);
+        a.p_pass = f64_pass_stride(H.p_len, ps.width);
+        a.tb_pass = f64_pass_stride(H.tb_len, ps.width);
+        a.slots_pass = PL.n_slots;
+        a.counters_pass = H.n_leaves;
         if (fac == 1)
-            launch_nr<1, uint16_t>(H, PL, a, nr, timed, st);
+            launch_nr<1, uint16_t>(H, PL, a, ps.width, timed, st);
         else
-            launch_nr<1, float>(H, PL, a, nr, timed, st);
+            launch_nr<1, float>(H, PL, a, ps.width, timed, st);
     }
 }
 
@@ -1931,7 +1993,7 @@ void build_product_plan(HMat& H, cudaStream_t st) {
     for (const LeafDesc& L : H.h_leaves) H.ld_max = std::max(H.ld_max, L.ld);
     for (int fac = 0; fac < 2; ++fac)
         if (has_factors(H, fac)) build_plan_for(H, H.plan[fac], fac == 1 ? 2 : 4, G, st);
-    H.counters.alloc(H.n_leaves);
+    H.counters.alloc((size_t)H.n_leaves * (16 / F64_PASS));  // per pass of a product
     HM_CUDA(cudaMemsetAsync(H.counters.p, 0, H.counters.bytes(), st));
     // single-RHS reduction order: blocks with many leaves of T first, factorless ones out
     std::vector<int32_t> big, small;
@@ -2067,10 +2129,19 @@ void ensure_product_scratch(HMat& H, int nrhs, cudaStream_t st) {
     H.nrhs_cap = cap;
 }
 
-int product_pass(int dtype) { return dtype == HM_F64 ? F64_PASS : 16; }
+int product_group(const HMat& H, int nr, int dtype) {
+    return dtype == HM_F64 ? f64_passes(H, nr).nrhs : std::min(nr, 16);
+}
+
+void product_split(HMat& H, const double* z, double* zs, int nr, cudaStream_t st) {
+    const F64Passes ps = f64_passes(H, nr);
+    k_gather_split<<<dim3((unsigned)ceil_div(H.ndof * ps.width, 256), ps.count), 256, 0, st>>>(
+        z, (float2*)zs, nullptr, H.N, nr, ps.width, f64_pass_stride(H.ndof, ps.width));
+    HM_LAUNCH_CHECK();
+}
 
 void product_core(HMat& H, const void* xc, void* yc, int nr, int dtype, int fac, cudaStream_t st, const int* skip) {
-    if (nr < 1 || nr > product_pass(dtype)) fail(HM_EINVAL, "product: too many right-hand sides in one pass");
+    if (nr < 1 || nr > product_group(H, nr, dtype)) fail(HM_EINVAL, "product: too many right-hand sides at once");
     ensure_product_scratch(H, nr, st);
     if (dtype == HM_F32 && padded_rhs(nr) != nr) {
         const int np = padded_rhs(nr);
@@ -2090,13 +2161,11 @@ void matvec(HMat& H, const void* x, void* y, int nrhs, int dtype, cudaStream_t s
     // FP32 factors when stored, unless the caller asks for a stored precision
     const int fac = factors == HM_BF16 ? 1 : (factors == HM_F32 ? 0 : (has_factors(H, 0) ? 0 : 1));
     if (!has_factors(H, fac)) fail(HM_EINVAL, "matvec: the requested factor precision is not stored");
-    const int pass = product_pass(dtype);
-    ensure_product_scratch(H, std::min(nrhs, pass), st);
-    for (int k0 = 0; k0 < nrhs; k0 += pass) {
-        const int nr = std::min(pass, nrhs - k0);
+    ensure_product_scratch(H, std::min(nrhs, 16), st);
+    for (int k0 = 0, nr = 0; k0 < nrhs; k0 += nr) {
+        // (16 right-hand sides are one group, so the next sixteen start a new one)
+        nr = product_group(H, std::min(nrhs - k0, 16 - k0 % 16), dtype);
         if (H.timing && k0 % 16 == 0) ++H.t_count;  // products of up to 16 right-hand sides
-        const int64_t tot = H.ndof * nr;
-        const unsigned gb = (unsigned)ceil_div(tot, 256);
         mark(H, 0, st);
         if (dtype == HM_F32) {
             const float* xf = (const float*)x + (int64_t)k0 * H.ndof;
@@ -2108,7 +2177,9 @@ void matvec(HMat& H, const void* x, void* y, int nrhs, int dtype, cudaStream_t s
         } else {
             const double* xd = (const double*)x + (int64_t)k0 * H.ndof;
             double* yd = (double*)y + (int64_t)k0 * H.ndof;
-            k_gather_split<<<gb, 256, 0, st>>>(xd, (float2*)H.xc.p, H.perm.p, H.N, nr);
+            const F64Passes ps = f64_passes(H, nr);
+            k_gather_split<<<dim3((unsigned)ceil_div(H.ndof * ps.width, 256), ps.count), 256, 0, st>>>(
+                xd, (float2*)H.xc.p, H.perm.p, H.N, nr, ps.width, f64_pass_stride(H.ndof, ps.width));
             mark(H, 1, st);
             run_core(H, H.xc.p, yd, nr, dtype, fac, true, st, nullptr, H.perm.p);
         }

@@ -927,17 +927,7 @@ __global__ void k_j3_apply(const float* __restrict__ j3, const double* __restric
     }
 }
 
-// interleave a set of FP64 vectors for the product: out[dof * nr + k] = in[k * ndof + dof]
-// F64 product operand: out[dof * nr + k] = (hi, lo) float split of in[k * ndof + dof]
-__global__ void k_interleave_split(const double* __restrict__ in, float2* __restrict__ out, int64_t ndof, int nr) {
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= ndof * nr) return;
-    const int64_t r = q / nr, k = q % nr;
-    const double v = in[k * ndof + r];
-    const float h = (float)v;
-    out[q] = make_float2(h, (float)(v - (double)h));
-}
-
+// interleave a set of vectors for the FP32 product: out[dof * nr + k] = in[k * ndof + dof]
 __global__ void k_to_f32_interleaved(const double* __restrict__ in, float* __restrict__ out, int64_t ndof, int nr) {
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= ndof * nr) return;
@@ -1462,7 +1452,7 @@ SolveWS& workspace(HMat& H, int nr, int m, cudaStream_t st) {
     W.bc.alloc(vn + VSLACK);
     W.corr.alloc(vn + VSLACK);
     W.y64.alloc(vn + VSLACK);
-    W.zi.alloc(vn + VSLACK);
+    W.zi.alloc((size_t)ceil_div(W.nr, 4) * 4 * H.ndof + 8 + VSLACK);  // as product_split asks
     W.dc.alloc(H.ndof + VSLACK);
     W.zf.alloc(vn + VSLACK);
     W.y32.alloc(vn + VSLACK);
@@ -1513,10 +1503,9 @@ unsigned g1(int64_t n) { return (unsigned)ceil_div(std::max<int64_t>(n, 1), 256)
 void apply_E(HMat& H, SolveWS& W, const double* z64, const float* z32, void* y, int nr, int dtype, int fac,
              cudaStream_t st, const int* skip = nullptr) {
     if (dtype == HM_F64) {
-        const int pass = product_pass(HM_F64);
-        for (int k0 = 0; k0 < nr; k0 += pass) {
-            const int nk = std::min(pass, nr - k0);
-            k_interleave_split<<<g1(H.ndof * nk), 256, 0, st>>>(z64 + k0 * H.ndof, (float2*)W.zi.p, H.ndof, nk);
+        for (int k0 = 0, nk = 0; k0 < nr; k0 += nk) {
+            nk = product_group(H, nr - k0, HM_F64);
+            product_split(H, z64 + k0 * H.ndof, W.zi.p, nk, st);
             product_core(H, W.zi.p, (double*)y + k0 * H.ndof, nk, HM_F64, fac, st, skip);
         }
     } else {
