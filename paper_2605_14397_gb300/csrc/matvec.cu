@@ -975,13 +975,15 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
             consumer_sync(NCW * 32);
             if (*s_flag) {
                 __threadfence();
-                for (int k = 0; k < nout; ++k)
-                    for (int r = threadIdx.x; r < rows; r += NCW * 32) {
-                        Vv s = 0;
-                        for (int p = 0; p < sp.nparts; ++p)
-                            s += __ldcg(slots + ((int64_t)(sp.slot_base + p) * NR + k) * a.ld_max + r);
-                        yc[out_at(k, r)] = s;
-                    }
+                // (over all right-hand sides at once: one after the other, 16 of an 84-row leaf
+                // were 16 rounds of load latencies for a sixth of the threads)
+                for (int e = threadIdx.x; e < nout * rows; e += NCW * 32) {
+                    const int k = NR == 1 ? 0 : e / rows, r = e - k * rows;
+                    Vv s = 0;
+                    for (int p = 0; p < sp.nparts; ++p)
+                        s += __ldcg(slots + ((int64_t)(sp.slot_base + p) * NR + k) * a.ld_max + r);
+                    yc[out_at(k, r)] = s;
+                }
                 if (threadIdx.x == 0) counters[cur] = 0;
             }
             consumer_sync(NCW * 32);
