@@ -148,7 +148,7 @@ template <class R>
 struct TensileEq {
     R tn, p0, p1, pn, chit;
     struct At {
-        R g, gx, n, ct, Tn;
+        R g, gx, n, ct, ict, Tn;
     };
     __device__ __forceinline__ At eval(const Law<R>& P, R x) const {
         At o;
@@ -157,9 +157,10 @@ struct TensileEq {
         root_of(p0 * p0 + p1 * p1 + o.n * o.n, v, inv);
         const bool ton = !(chit >= v);
         o.ct = ton ? v : chit;
+        o.ict = ton ? inv : R(0);
         o.Tn = tn - P.Kn * x;
         o.g = o.Tn - P.st(o.ct, st1);
-        o.gx = -P.Kn - st1 * (ton ? o.n * inv : R(0));
+        o.gx = -P.Kn - st1 * (o.n * o.ict);
         return o;
     }
 };
@@ -262,6 +263,13 @@ __device__ __forceinline__ double inverse_slope(double x, double gx, int* st) {
         return 0.0;
     }
     return 1.0 / gx;
+}
+
+// An internal variable as it leaves the step: where it grew (inv = 1/v is not 0) v = q inv
+// carries the rounding of both factors, and one Newton step takes it to that of sqrt(q)
+// (1,000,000 points of a softening joint: 24 us more with square roots, 10 with this).
+__device__ __forceinline__ double grown(double inv, double q, double v) {
+    return inv > 0.0 ? fma(0.5 * inv, fma(-v, v, q), v) : v;
 }
 
 // open state: T' = 0, all of dd + C^-1 T'^n inelastic
@@ -375,8 +383,8 @@ __device__ __forceinline__ void finish_coulomb(const Prm& P, const Law<double>& 
     r.dp[0] = o.a;
     r.dp[1] = o.b;
     r.dp[2] = o.n;
-    r.chis = o.cs;
-    r.chit = o.ct;
+    r.chis = grown(o.ics, o.a * o.a + o.b * o.b, o.cs);
+    r.chit = grown(o.ict, o.a * o.a + o.b * o.b + o.n * o.n, o.ct);
     r.wdil = p.wdil + o.psi * x;
     r.mode = M_COULOMB;
     if (!want_cep) return;
@@ -409,7 +417,7 @@ __device__ __forceinline__ void finish_apex(const Prm& P, const Law<double>& W, 
     double v, inv, f1;
     root_of(e.a * e.a + e.b * e.b, v, inv);
     const bool on = !(p.chis >= v);
-    r.chis = on ? v : p.chis;
+    r.chis = on ? grown(inv, e.a * e.a + e.b * e.b, v) : p.chis;
     e.f = W.f(r.chis, f1) + W.fr;
     e.tn = Ttr[2];
     e.pn = dpb[2];
@@ -424,7 +432,7 @@ __device__ __forceinline__ void finish_apex(const Prm& P, const Law<double>& W, 
     r.dp[0] = e.a;
     r.dp[1] = e.b;
     r.dp[2] = o.n;
-    r.chit = o.ct;
+    r.chit = grown(o.ict, e.a * e.a + e.b * e.b + o.n * o.n, o.ct);
     r.wdil = p.wdil;
     r.mode = M_APEX;
     if (!want_cep) return;
@@ -454,7 +462,7 @@ __device__ __forceinline__ void finish_tensile(const Prm& P, const Law<double>& 
     r.dp[1] = dpb[1];
     r.dp[2] = o.n;
     r.chis = p.chis;
-    r.chit = o.ct;
+    r.chit = grown(o.ict, e.p0 * e.p0 + e.p1 * e.p1 + o.n * o.n, o.ct);
     r.wdil = p.wdil;
     r.mode = M_TENSILE;
     if (!want_cep) return;
