@@ -190,7 +190,8 @@ def _coulomb(P, Ttr, dp, chis, chit, wdil):
         return tau1 + friction(P, chis1) * Tn1 - cohesion(P, chit1)
 
     hi = tau_tr.real / P.Ks
-    if g(hi).real > 0.0:
+    chis1, chit1, _, _, _, Tn1 = state(hi)
+    if (friction(P, chis1) * Tn1 - cohesion(P, chit1)).real > 0.0:  # g(hi), where tau1 is zero by definition
         return _apex(P, Ttr, dp, chis, chit, wdil)
     dl = _root(g, hi)
     chis1, chit1, psi1, dp1, tau1, Tn1 = state(dl)

@@ -99,7 +99,7 @@ struct CoulombEq {
     R tau, itau, s0, s1, tn, p0, p1, pn, chis, chit;
     struct At {
         R g, gx;
-        R a, b, n, cs, ct, psi, f, ta, Tn;  // inelastic DD, internal variables, strengths, tractions
+        R a, b, n, cs, ct, psi, f, c, ta, Tn;  // inelastic DD, internal variables, strengths, tractions
         R ics, ict, f1, psi1, c1;           // 1/cs and 1/ct where they grow (else 0); slopes of f, psi, c
     };
     __device__ __forceinline__ At eval(const Law<R>& P, R x) const {
@@ -119,10 +119,10 @@ struct CoulombEq {
         const bool ton = !(chit >= v);
         o.ct = ton ? v : chit;
         o.ict = ton ? inv : R(0);
-        const R c = P.c(o.ct, o.c1);
+        o.c = P.c(o.ct, o.c1);
         o.ta = tau - P.Ks * x;
         o.Tn = tn - P.Kn * (o.psi * x);
-        o.g = o.ta + o.f * o.Tn - c;
+        o.g = o.ta + o.f * o.Tn - o.c;
         o.gx = slope(P, o, x, R(1), o.a * s0 + o.b * s1, -P.Ks, R(0));
         return o;
     }
@@ -360,7 +360,10 @@ __device__ __forceinline__ int classify(const Prm& P, const Law<double>& W, cons
     }
     if (kind == M_COULOMB) {
         if (!(tau > 0.0)) return M_APEX;
-        if (make_coulomb<double, true>(tau, Ttr, dpb, p).eval(W, tau * P.iKs).g > 0.0) return M_APEX;
+        // g where the shear traction vanishes: without ta, which is rounding noise there and would
+        // decide for a frictionless contact (f = c = 0: g is zero), an apex return that opens it
+        const auto o = make_coulomb<double, true>(tau, Ttr, dpb, p).eval(W, tau * P.iKs);
+        if (o.f * o.Tn - o.c > 0.0) return M_APEX;
     }
     return kind;
 }

@@ -55,3 +55,33 @@ def test_grown_internal_variables_are_rounded_square_roots(name):
             assert np.sqrt((err ** 2).mean()) <= 0.58, (kind, c, np.sqrt((err ** 2).mean()))
             tested += 1
     assert tested >= 2
+
+
+@pytest.mark.parametrize("Ks", [7.0, 10.0, 1.0 / 3.0, 13.7])
+@pytest.mark.parametrize("fp", [0.0, 0.4])
+def test_frictionless_contact_slips(Ks, fp):
+    """A pre-existing fracture without friction (or softened to none by the step's slip) under
+    compression: g is zero where the shear traction vanishes, and the return is the Coulomb one
+    with all of the trial shear inelastic, never an open state.  Bars: a few roundings of the
+    trial and shear tractions, of the slip and of K_s."""
+    rng = np.random.default_rng(int(100 * Ks) + int(10 * fp))
+    n = 20000
+    kw = dict(Ks=Ks, Kn=2 * Ks, fp=fp, fr=0.0, psip=0.0, dc=1e-6 if fp else 0.2, cp=0.0, sigp=0.0, wc=0.0, alphaR=0.0)
+    T = np.c_[rng.normal(size=(n, 2)) * 0.2, -rng.uniform(0.5, 1.5, n)]
+    dp, chi = np.zeros((n, 3)), np.zeros((n, 3))
+    dd = np.c_[rng.normal(size=(n, 2)) * 0.08, rng.normal(size=n) * 1e-3]
+    tr = T + np.array([Ks, Ks, 2 * Ks]) * dd
+    tau = np.hypot(tr[:, 0], tr[:, 1])
+    assert (tr[:, 2] < 0).all() and (tau > 1.1 * fp * np.abs(tr[:, 2])).sum() > 1000
+    T1, dp1, chi1, cep, mode, cnt = update(kw, (T, dp, chi, dd))
+    slips = tau > 1.1 * fp * np.abs(tr[:, 2]) + 2 * Ks * kw["dc"] * (fp > 0)
+    u = 2.0 ** -53
+    assert (mode[slips] == I.COULOMB).all() and cnt[3] == cnt[4] == cnt[5] == 0
+    assert (np.abs(T1[slips, :2]).max(axis=1) <= 16 * u * tau[slips]).all()
+    assert np.abs(T1[slips, 2] - tr[slips, 2]).max() <= 8 * u * 2
+    trial = 4 * u * (np.abs(T) + Ks * np.abs(dd))[:, :2].max(axis=1)  # the trial traction's own roundings
+    assert (np.abs(dp1[slips, :2] - tr[slips, :2] / Ks).max(axis=1) <= (16 * u * tau + trial)[slips] / Ks).all()
+    assert np.abs(cep[slips][:, :2, :2]).max() <= 64 * u * Ks and np.abs(cep[slips, 2, 2] - 2 * Ks).max() <= 8 * u * 2 * Ks
+    P = I.Params(**kw)
+    q = np.flatnonzero(slips)[:150]
+    assert np.array_equal(mode[q], [I.update(P, T[e], dp[e], chi[e], dd[e])["mode"] for e in q])
