@@ -207,7 +207,7 @@ def time_gmres(H, el, dev, torch, reps=3):
 def run_faults64(args, dev, torch, hmat, synth):
     """64 independent disk faults (log-uniform 2k-40k elements, seeded normals and nu,
     795,192 elements in all): one batched H-matrix (one work list, 4 launches per
-    product; also replayed from a CUDA graph) against per-fault products (64 x 5
+    product; also replayed from a CUDA graph) against per-fault products (64 x 4
     launches; also 64 graph replays).  value = algorithmic bytes of all 64 products /
     time of the batched product."""
     import numpy as np
@@ -305,9 +305,8 @@ def run_faults64(args, dev, torch, hmat, synth):
                        "l2": "operator %.1f GB >> 129 MB L2: no flush" % (Bytes / 1e9)},
             "frac_of_hbm_peak": value / hbm, "peak_source": peak_kind,
             "ms_per_product": res, "speedup_batched_over_per_fault": res["per_fault"] / best_ms,
-            "launches_per_product": {"batched": 5, "per_fault": 5 * len(parts)}, "clocks": clocks,
-            "batched_phases_ms": {k: ph[k] / max(ph["count"], 1) for k in ("gather", "phase1", "reduce", "phase2",
-                                                                           "scatter")}}
+            "launches_per_product": {"batched": 4, "per_fault": 4 * len(parts)}, "clocks": clocks,
+            "batched_phases_ms": {k: ph[k] / max(ph["count"], 1) for k in ("gather", "phase1", "reduce", "phase2")}}
     if args.tune:
         line["autotune_largest_fault"] = hmat.autotune(els[int(np.argmax(Ns))], E, float(nus[int(np.argmax(Ns))]),
                                                        eps, "f32", leaves=(32, 48, 64, 96, 128), etas=(2.0,),
@@ -364,7 +363,7 @@ def run_planes(args, dev, torch, hmat, synth):
             H.timing(False)
             ph = H.timing_read()
             phases["%s_%drhs" % (fac, nrk)] = {k: ph[k] / max(ph["count"], 1)
-                                               for k in ("gather", "phase1", "reduce", "phase2", "scatter")}
+                                               for k in ("gather", "phase1", "reduce", "phase2")}
     clocks = sampler.stop()
     H.check(stream)
     # algorithmic bytes of one 16-RHS product: every stored near entry (4 B) and factor
@@ -980,7 +979,7 @@ def main():
                 "unit": "GB/s", "frac": ach / hbm, "peak_source": peak_kind,
                 "traffic": recorded_traffic("k_phase2"),
                 "algorithmic_bytes_per_launch": B2, "launch_ms": t2 * 1e3,
-                "phases_ms": {k: ph[k] / cnt for k in ("gather", "phase1", "reduce", "phase2", "scatter")},
+                "phases_ms": {k: ph[k] / cnt for k in ("gather", "phase1", "reduce", "phase2")},
                 "phase1_GBs": B1 / t1 / 1e9 if t1 > 0 else None}
 
     # the compensated product (FP64 vectors, the same FP32 factors): the operator of the

@@ -458,8 +458,8 @@ hm_status hm_coupled_solve(const hm_hmat* h, const hm_flow* f, const double* k_d
  *   t^(n+1) (backward Euler, like f, psi, c, sigma_t in the return);
  *   mode at the trial state with the strengths of t^n: elastic if F_c <= 0 and F_t <= 0,
  *   else Coulomb if h = |tau| - (c - f sigma_t) - (sqrt(1 + f^2) - f)(T'_n - sigma_t) > 0,
- *   else tensile; a Coulomb return with no root before tau = 0 returns to the cone's apex
- *   (tau = 0, f T'_n = c, shear fully inelastic);
+ *   else tensile; a Coulomb return with no root before tau = 0 (f T'_n > c there) returns
+ *   to the cone's apex (tau = 0, f T'_n = c, shear fully inelastic);
  *   full damage when wc = 0 (pre-existing fracture) or chi_t >= wc: a fully damaged
  *   point with a tensile trial traction is open (T' = 0, C^ep = 0, Delta delta + C^-1 T'^n
  *   inelastic); otherwise it is in contact with its normal inelastic DD at
@@ -467,9 +467,10 @@ hm_status hm_coupled_solve(const hm_hmat* h, const hm_flow* f, const double* k_d
  *   tensile or apex return that reaches full damage ends open;
  *   w_dil (the dilatant part of w_R) grows by psi dl in every Coulomb return.
  * The plastic multiplier solves a scalar equation (Newton safeguarded by bisection);
- * parameters must keep it monotone (interface stiffness above the softening rates).
- * C^ep is exact within the active mode (forward-mode dual numbers and the implicit
- * function theorem at the multiplier's root).
+ * parameters must keep it monotone (interface stiffness above the softening rates): where
+ * it has several roots, which one is returned is unspecified.  C^ep is exact within the
+ * active mode (closed-form derivatives and the implicit function theorem at the
+ * multiplier's root).
  * Arrays (device, n points, row-major): T_dev, dp_dev (n x 3: T'^n and delta^p_n),
  * chi_dev (n x 3: chi_s, chi_t, w_dil), dd_dev (n x 3: Delta delta) in; T1_dev, dp1_dev,
  * chi1_dev (n x 3) out, each may be the same array as its input; cep_dev (n x 9, row i =

@@ -194,8 +194,8 @@ void graphs_clear(HMat& H) {
     H.graphs.clear();
 }
 
-// y = E x through a CUDA graph of the whole product (gather, the three streaming
-// kernels, scatter), instantiated on first use for this (x, y, nrhs, dtype) and
+// y = E x through a CUDA graph of the whole product (gather, phase 1, reduction, phase 2),
+// instantiated on first use for this (x, y, nrhs, dtype) and
 // replayed on `st` afterwards: one launch of host work per product.
 void matvec_graph(HMat& H, const void* x, void* y, int nrhs, int dtype, cudaStream_t st) {
     if (H.timing) {  // per-phase events cannot live inside a replayed graph

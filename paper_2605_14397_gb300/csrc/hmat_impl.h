@@ -14,8 +14,7 @@
 //   gather     xc = x[perm]                       (cluster order, RHS interleaved)
 //   phase 1    P = V_t^T xc_t                      per leaf t (one partial per V column)
 //   reduce     tb_b = sum over the leaves t of T_b of the partials of b
-//   phase 2    yc_s = [D_s | U_s] z_s,  z = xc (near columns) or tb (U columns)
-//   scatter    y[perm] = yc
+//   phase 2    y[perm]_s = [D_s | U_s] z_s,  z = xc (near columns) or tb (U columns)
 // A near tile, a U slice and a V slice each read (or write) a contiguous range of
 // xc / tb / P, so the operands of a pipeline chunk are one bulk copy.
 #pragma once

@@ -12,9 +12,9 @@
 // columns) and the chunk list is split into equal byte ranges, one per CTA ("stream-K"):
 // every SM streams the same number of bytes.  One producer thread moves each chunk --
 // its coefficients and, in phase 2, the contiguous range of operands it multiplies --
-// with two cp.async.bulk (TMA) copies into a 4-stage shared-memory ring guarded by
-// mbarriers; 8 or 16 consumer warps each take columns of the chunk, lanes over rows,
-// and touch no global memory except at leaf boundaries.  A row leaf whose columns fall
+// with two cp.async.bulk (TMA) copies into a shared-memory ring of four stages (six in
+// k_phase1_mr and some tile shapes) guarded by mbarriers; 8 to 16 consumer warps each take
+// columns of the chunk, lanes over rows, and touch no global memory except at leaf boundaries.  A row leaf whose columns fall
 // into several CTAs is finished by the last of them (atomic arrival count, partials
 // summed in CTA order), so the result is deterministic.
 //
@@ -1147,9 +1147,10 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase2(StreamArgs a) {
     if (cur >= 0) flush();
 }
 
-// ---- phase 1: P = V_t^T xc_t, one partial per V column (F32 mode, 1 to 4 right-hand sides)
+// ---- phase 1: P = V_t^T xc_t, one partial per V column (F32 mode, 1 or 4 right-hand sides)
 template <class C, int NR, int RPL, int NCW, int ST = STAGES>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
+    static_assert(NR == 1 || NR == 4, "one right-hand side, or four in pairs");
     using Acc = float;
     using Vv = float;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -1258,13 +1259,8 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
             for (int ii = 0; ii < RPL; ++ii) {
                 const int r = lane + 32 * ii;
                 const float v = r < rows ? coef(col, r) : 0.f;
-                if constexpr (std::is_same<Acc, float>::value && NR % 2 == 0) {
 #pragma unroll
-                    for (int k = 0; k < NR; k += 2) acc_fma2(acc[k], acc[k + 1], v, xr[k][ii], xr[k + 1][ii]);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < NR; ++k) acc_fma(acc[k], v, xr[k][ii]);
-                }
+                for (int k = 0; k < NR; k += 2) acc_fma2(acc[k], acc[k + 1], v, xr[k][ii], xr[k + 1][ii]);
             }
             const int k = warp_reduce_scatter<NR>(acc, lane);
             if ((lane & (32 / NR - 1)) == 0) P[(ch.zoff + c) * NR + k] = (Vv)acc_value(acc[0]);
@@ -1714,7 +1710,7 @@ void timing_accumulate(HMat& H) {
     H.ev_used = 0;
 }
 
-// phase boundary idx (0 before the gather ... 5 after the scatter) of one product
+// phase boundary idx (0 before the gather, 4 and 5 after phase 2) of one product
 void mark(HMat& H, int idx, cudaStream_t st) {
     if (!H.timing) return;
     if (idx == 0 && H.ev_used + EV_PER_PRODUCT > (int)H.ev.size()) timing_accumulate(H);
@@ -1723,8 +1719,10 @@ void mark(HMat& H, int idx, cudaStream_t st) {
 }
 
 // consumer warps of phase 1 and phase 2, and phase 2's row split, per right-hand-side
-// count: as many warps as the per-thread registers (accumulators and operands) allow
-// phase 2's row split: two or three row blocks per warp with 16 RHS, else (one F32 RHS apart)
+// count: as many warps as the per-thread registers (accumulators and operands) allow.
+// (Left spilling: k_phase1_f64 with three or four right-hand sides on leaves above 64 elements,
+// 140 to 292 bytes of its operands, and the BF16 16-RHS phase 2 on 192-row leaves, 56 bytes.)
+// Phase 2's row split: two or three row blocks per warp with 16 RHS, else (one F32 RHS apart)
 // six
 template <int MODE>
 constexpr int rs_for(int NR, int RPL) {
@@ -1843,10 +1841,9 @@ template <int MODE, class C, int NR, bool TC = true, bool PASSES = false>
 void launch_rpl(HMat& H, const HMat::Plan& PL, const StreamArgs& a, bool timed, cudaStream_t st) {
     // 16 RHS split a column's rows over two warps, so leaves of at most 128 rows have a
     // variant of their own: with three row blocks a warp, one of 99 rows left the second warp
-    // one block (three 150 x 150 planes, BF16: phase 2 905 us before, 692 with two and
-    // two and the finer tensor-core mapping;
-    // a split computed from each leaf's rows cost the 176-row leaves of three 100 x 100 planes
-    // 10 %)
+    // one block (three 150 x 150 planes, BF16: phase 2 1,175 us, 905 with exact counts, 692 with
+    // two blocks and two and the finer tensor-core mapping; a split computed from each leaf's
+    // rows cost the 176-row leaves of three 100 x 100 planes 10 %)
     if (NR == 16 && H.ld_max <= 128) {
         if constexpr (NR == 16) launch_phases<MODE, C, NR, 4, STAGES, 0, 0, TC, PASSES>(H, PL, a, timed, st);
     } else if (H.ld_max <= 192)

@@ -220,8 +220,8 @@ __global__ void __launch_bounds__(512) k_bj_build(const LeafDesc* __restrict__ l
 // coefficients of unknown k against equations p_0 .. p_(n-1), so A^-1[k][m] = W[p_k][q]
 // with p_q = m.
 //
-// The sweeps go in panels of BJR_PB columns.  The last warp sweeps a panel's own columns in
-// its registers and leaves the multipliers c_k[i] (column k as step k found it), the pivots
+// The sweeps go in panels of BJR_PB columns.  The last warp sweeps a panel's own columns (rows
+// of eight in shared memory, a lane's rows in registers for a step) and leaves the multipliers c_k[i] (column k as step k found it), the pivots
 // and their rows; the other warps carry the pivot rows of the remaining columns through the
 // panel (a thread per column), bring the next panel's columns up to date for the last warp,
 // and apply the panel's rank-1 updates to their tiles while it sweeps.  Each entry sees the
@@ -434,7 +434,7 @@ __device__ __forceinline__ bool bjr_matrix_warps(float (&A)[AR][BC], BjrShared<A
         const int buf = P & 1, pb = min(BJR_PB, n - k0);
         rows(buf, pb, std::true_type{});
         __syncthreads();
-        // the pivot rows through the panel, a thread per column (past the last step: r = 0)
+        // the pivot rows through the panel, a thread per column (a partial last panel ends at pb)
         if (t < 32 * BC) {
             float v[BJR_PB];
 #pragma unroll

@@ -489,7 +489,8 @@ class HMatrix:
         _check(lib().hm_hmat_timing(self.handle, 1 if enable else 0))
 
     def timing_read(self):
-        """Milliseconds summed per phase: gather, phase1, reduce, phase2, scatter, count."""
+        """Milliseconds summed per phase: gather, phase1, reduce, phase2, count; scatter is the
+        end of the product, where no kernel runs any more (phase 2 writes user order)."""
         out = (ctypes.c_double * 6)()
         _check(lib().hm_hmat_timing_read(self.handle, out))
         return dict(gather=out[0], phase1=out[1], reduce=out[2], phase2=out[3], scatter=out[4], count=int(out[5]))
