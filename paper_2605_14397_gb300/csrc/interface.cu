@@ -602,10 +602,10 @@ __global__ void __launch_bounds__(128) k_iface_classify(IfArgs a) {
     flush_counts(a, s_cnt);
 }
 
-// Pass 2: the listed points of one return kind, grid-stride.  Bound by the FP64 pipe (80 %
-// busy).  Of 1,000,000 points of a softening joint with the tangent, the Coulomb returns
-// take 0.47 ms (dual numbers: 7.44), the apex returns 0.15 (1.42), the tensile ones 0.03
-// (0.48), the classification 0.20 (0.32); the whole update 0.84 ms (9.55).
+// Pass 2: the listed points of one return kind, grid-stride.  Bound by the FP64 pipe (80 to
+// 86 % busy).  Of 1,000,000 points of a softening joint with the tangent, the Coulomb returns
+// take 0.49 ms (dual numbers: 7.44), the apex returns 0.15 (1.42), the tensile ones 0.02
+// (0.48), the classification 0.20 (0.32); the whole update 0.87 ms (9.56).
 template <int KIND>
 __global__ void __launch_bounds__(128) k_iface_return(IfArgs a) {
     __shared__ unsigned int s_cnt[N_MODES + 1];

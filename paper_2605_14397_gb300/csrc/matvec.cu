@@ -56,7 +56,7 @@ struct FF2 {
 // right-hand side, so from four on the pass is bound by the FP32 pipe and streaming the
 // coefficients again for the next four costs less than the registers of a wider pass:
 // six RHS of a 12,892-element fault (615 MB of coefficients) took 2.82 ms in one pass of a
-// 16-wide kernel that spilled, 0.56 ms in two passes of three (f64_passes).
+// 16-wide kernel that spilled, 0.55 ms in two passes of three (f64_passes).
 constexpr int F64_PASS = 4;
 
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
