@@ -14,9 +14,9 @@
 // its coefficients and, in phase 2, the contiguous range of operands it multiplies --
 // with two cp.async.bulk (TMA) copies into a shared-memory ring of four stages (six in
 // k_phase1_mr and some tile shapes) guarded by mbarriers; 8 to 16 consumer warps each take
-// columns of the chunk, lanes over rows, and touch no global memory except at leaf boundaries.  A row leaf whose columns fall
-// into several CTAs is finished by the last of them (atomic arrival count, partials
-// summed in CTA order), so the result is deterministic.
+// columns of the chunk, lanes over rows, and touch no global memory except at leaf
+// boundaries.  A row leaf whose columns fall into several CTAs is finished by the last of
+// them (atomic arrival count, partials summed in CTA order), so the result is deterministic.
 //
 // Arithmetic modes over the same FP32/BF16 coefficient streams:
 //   F32: float vectors, FP32 accumulation;
@@ -1283,8 +1283,8 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) k_phase1(StreamArgs a) {
 // x past the leaf's rows is zero, and everything an unchecked read can reach is
 // finite (the ring is zeroed first), so nothing is bound-checked.  Columns are dealt in units
 // of 4 CL across chunks; the ring is six deep because the warps work on about three chunks
-// at a time.  16 RHS take eight warps: 64 accumulators and their operands a lane.  Bound by the FP32 pipe and shared-memory reads: 16 RHS on three 100 x 100 planes
-// (0.82 GB of V, 0.12 ms at the copy bandwidth): 0.38 ms a column at a time, 0.21 ms now.
+// at a time.  16 RHS take eight warps: 64 accumulators and their operands a lane.  Bound by
+// the FP32 pipe and shared-memory reads: 16 RHS on three 100 x 100 planes (0.82 GB of V, 0.12 ms at the copy bandwidth): 0.38 ms a column at a time, 0.21 ms now.
 template <class C>
 __device__ __forceinline__ float4 coef4(const C* p);
 template <>
@@ -1832,7 +1832,8 @@ void launch_phases(HMat& H, const HMat::Plan& PL, const StreamArgs& base, bool t
     a.cta_begin = PL.cta2.p;
     a.split = PL.split.p;
     a.wait_x = !(H.n_far > 0 && H.p_len > 0);
-    launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC, PASSES>, dim3(H.grid, passes), dim3((NCW2 + 1) * 32), smem2, st, a);
+    launch_pdl(k_phase2<MODE, C, NR, RPL, NCW2, RS, ST, TC, PASSES>, dim3(H.grid, passes), dim3((NCW2 + 1) * 32), smem2,
+               st, a);
     HM_LAUNCH_CHECK();
     if (timed) mark(H, 4, st);
 }
